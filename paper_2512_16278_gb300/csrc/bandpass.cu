@@ -261,9 +261,9 @@ __global__ void __launch_bounds__(kArThreads, 1) arpls_kernel(ArplsArgs g) {
 }
 
 // y[(I * N + a) * n_chan + j]: mean of beam a, channel j over interval I,
-// from the Gram sums (public [cell][P] or interleaved [cell/8][P][8]).
-__global__ void bandpass_input_kernel(const int64_t* __restrict__ sums, int interleaved,
-                                      int n_beam, int n_chan, int n_sub, int interval, int psum,
+// from the Gram sums [cell][P].
+__global__ void bandpass_input_kernel(const int64_t* __restrict__ sums, int n_beam, int n_chan,
+                                      int n_sub, int n_samp_sub, int interval, int psum,
                                       double* __restrict__ y, int64_t total) {
   const int N1 = n_beam + 1;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -273,24 +273,16 @@ __global__ void bandpass_input_kernel(const int64_t* __restrict__ sums, int inte
     const int a = (int)(ia % n_beam);
     const int I = (int)(ia / n_beam);
     const int e_sa = a * N1 - a * (a - 1) / 2 + (n_beam - a);  // S_a
-    const int e_n = psum - 1;                                   // n
     const int k0 = I * interval;
     const int k1 = k0 + interval < n_sub ? k0 + interval : n_sub;
-    int64_t s = 0, nn = 0;
-    for (int k = k0; k < k1; ++k) {
-      const int64_t cell = (int64_t)k * n_chan + j;
-      const int64_t* src = interleaved ? sums + (cell >> 3) * psum * 8 + (cell & 7) : sums + cell * psum;
-      const int step = interleaved ? 8 : 1;
-      s += src[(int64_t)e_sa * step];
-      nn += src[(int64_t)e_n * step];
-    }
-    y[idx] = (double)s / (double)nn;
+    int64_t s = 0;
+    for (int k = k0; k < k1; ++k) s += sums[((int64_t)k * n_chan + j) * psum + e_sa];
+    y[idx] = (double)s / (double)((int64_t)(k1 - k0) * n_samp_sub);
   }
 }
 
 // One warp per cell: C_ab = cov_ab / n^2 + d_a d_b, packed upper triangle.
-__global__ void ccm_bandpass_kernel(const int64_t* __restrict__ sums, int interleaved,
-                                    int64_t n_cells, int n_beam, int n_chan, int interval,
+__global__ void ccm_bandpass_kernel(const int64_t* __restrict__ sums, int64_t n_cells, int n_beam, int n_chan, int interval,
                                     int psum, int np, const double* __restrict__ z,
                                     float* __restrict__ ccm) {
   extern __shared__ unsigned char bp_raw[];
@@ -302,13 +294,8 @@ __global__ void ccm_bandpass_kernel(const int64_t* __restrict__ sums, int interl
   const int64_t cell = (int64_t)blockIdx.x * warps + warp;
   if (cell >= n_cells) return;
   const int N1 = n_beam + 1;
-  if (interleaved) {
-    const int64_t* src = sums + (cell >> 3) * psum * 8 + (cell & 7);
-    for (int e = lane; e < psum; e += 32) S[e] = src[(int64_t)e * 8];
-  } else {
-    const int64_t* src = sums + cell * psum;
-    for (int e = lane; e < psum; e += 32) S[e] = src[e];
-  }
+  const int64_t* src = sums + cell * psum;
+  for (int e = lane; e < psum; e += 32) S[e] = src[e];
   __syncwarp();
   const int64_t n = S[psum - 1];
   const int k = (int)(cell / n_chan), j = (int)(cell % n_chan);
@@ -377,21 +364,19 @@ cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_bandpass_input(const mraid_plan_s* pl, const int64_t* d_sums, bool interleaved,
-                                  int interval, double* d_y) {
+cudaError_t launch_bandpass_input(const mraid_plan_s* pl, const int64_t* d_sums, int interval, double* d_y) {
   const int n_int = (pl->p.n_sub + interval - 1) / interval;
   const int64_t total = (int64_t)n_int * pl->p.n_beam * pl->p.n_chan;
   int64_t blocks = (total + 255) / 256;
   if (blocks > (int64_t)pl->sm_count * 16) blocks = (int64_t)pl->sm_count * 16;
   if (blocks < 1) return cudaSuccess;
   bandpass_input_kernel<<<(unsigned)blocks, 256, 0, pl->stream>>>(
-      d_sums, interleaved ? 1 : 0, pl->p.n_beam, pl->p.n_chan, pl->p.n_sub, interval, pl->psum,
+      d_sums, pl->p.n_beam, pl->p.n_chan, pl->p.n_sub, pl->p.n_samp_sub, interval, pl->psum,
       d_y, total);
   return cudaGetLastError();
 }
 
-cudaError_t launch_ccm_bandpass(const mraid_plan_s* pl, const int64_t* d_sums, bool interleaved,
-                                int interval, const double* d_z, float* d_ccm) {
+cudaError_t launch_ccm_bandpass(const mraid_plan_s* pl, const int64_t* d_sums, int interval, const double* d_z, float* d_ccm) {
   const int psum = pl->psum;
   int warps = (int)(40960 / ((size_t)psum * 8 + kMaxBeam * 4));
   warps = warps < 1 ? 1 : (warps > 8 ? 8 : warps);
@@ -402,7 +387,7 @@ cudaError_t launch_ccm_bandpass(const mraid_plan_s* pl, const int64_t* d_sums, b
   const int64_t blocks = (pl->n_cells + warps - 1) / warps;
   if (blocks > 0)
     ccm_bandpass_kernel<<<(unsigned)blocks, warps * 32, smem, pl->stream>>>(
-        d_sums, interleaved ? 1 : 0, pl->n_cells, pl->p.n_beam, pl->p.n_chan, interval, psum,
+        d_sums, pl->n_cells, pl->p.n_beam, pl->p.n_chan, interval, psum,
         pl->np, d_z, d_ccm);
   return cudaGetLastError();
 }
@@ -524,21 +509,20 @@ mraid_status mraid_run_bandpass(mraid_plan_t pl, const void* d_data,
   }
   e = cudaMemsetAsync(pl->d_sweeps, 0, 3 * sizeof(unsigned long long), pl->stream);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
-  bool inter = false;
-  st = gram_sums_pass(pl, d_data, nullptr, &inter);
+  st = ccm_range(pl, d_data, 0, pl->p.n_sub, pl->ws.sums, nullptr);
   if (st != MRAID_OK) return st;
   // the sums pass may count zero-variance beams; nothing is normalised here
   e = cudaMemsetAsync(pl->d_degenerate, 0, sizeof(unsigned long long), pl->stream);
   if (e == cudaSuccess)
     e = MRAID_PROF(pl, K_BP_INPUT,
-                   launch_bandpass_input(pl, pl->ws.sums, inter, interval, pl->bp_y));
+                   launch_bandpass_input(pl, pl->ws.sums, interval, pl->bp_y));
   if (e == cudaSuccess)
     e = MRAID_PROF(pl, K_ARPLS,
                    launch_arpls(pl, pl->bp_y, n_sys, pl->p.n_chan, bp->lam, bp->ratio,
                                 bp->itermax, pl->bp_z, d_bandpass, pl->bp_iters, pl->ar_work));
   if (e == cudaSuccess)
     e = MRAID_PROF(pl, K_CCM_BP,
-                   launch_ccm_bandpass(pl, pl->ws.sums, inter, interval, pl->bp_z, pl->ws.corr));
+                   launch_ccm_bandpass(pl, pl->ws.sums, interval, pl->bp_z, pl->ws.corr));
   if (e != cudaSuccess) return cuda_fail(e, "bandpass kernels");
   e = MRAID_PROF(pl, K_EIG, launch_eig(pl, pl->ws.corr, pl->n_cells, d_evals, d_q1, d_stat));
   if (e != cudaSuccess) return cuda_fail(e, "eig launch");

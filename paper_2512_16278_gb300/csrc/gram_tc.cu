@@ -1,36 +1,28 @@
-// gram_tc.cu - exact augmented Gram sums of 8-bit multi-beam data on the
-// 5th-generation tensor cores (tcgen05), fused with the correlation.
+// gram_tc.cu - two inputs on the 5th-generation tensor cores (tcgen05), each
+// fused with the correlation (Section 3.2, Eq. 1): the total power of two
+// 8-bit polarisations (exact sums), and float32 samples.
 //
-// Section 3.2, Eq. 1. For a cell (channel j, sub-integration k) with
-// samples x_b(t), the kernel forms G = Y~ Y~^T with Y~ = [x - 128; 1]:
-// the centred values x - 128 are exact in f16, every product is an integer
-// of magnitude <= 2^14 and every partial sum over <= 1024 samples is an
-// integer of magnitude <= 2^24, so the FP32 tensor-core accumulation is
-// exact. From the centred sums, cov_ab = n G_ab - G_a G_b is exact in int64
-// (it does not depend on the centring) and r_ab = cov_ab / sqrt(var_a var_b)
-// is rounded to float once. The raw uint8 sums, when requested, follow from
-// S_ab = G_ab + 128 (G_a + G_b) + 128^2 n and S_a = G_a + 128 n.
-//
-// Data flow per persistent CTA (one per SM), warp-specialised:
-//   warp 0    TMA: box {16 channels, 32 samples, N beams} of u8 into a ring
-//             as deep as shared memory allows (cp.async.bulk.tensor, mbarrier
-//             transaction count), so streaming continues through epilogues;
-//   warps 4-7 convert each box to centred f16 operand tiles in the
-//             MN-major canonical layout (8 channels x 8 samples per core
-//             matrix) into a 2-deep ring. A slot is one beam (slot N is the
-//             row of ones) across the 8 channels of a group; the slots are
-//             laid out as [g0 0..15][g0 16..N][g1 16..N][g1 0..15];
+// Two polarisations: x = p0 + p1 (0..510); x - 255 is exact in f16, products
+// reach 2^16, so TMEM accumulates pieces of <= 256 samples exactly and the
+// epilogue adds the pieces as integers. Data flow per persistent CTA (one
+// per SM), warp-specialised:
+//   warp 0    TMA: box {16 channels, 64 samples, 2N blocks} of u8 into a ring
+//             as deep as shared memory allows;
+//   warps 4-7 add the polarisations and convert to centred f16 operand tiles
+//             in the MN-major canonical layout (8 channels x 8 samples per
+//             core matrix) in a 2-deep ring. A slot is one beam (slot N is
+//             the row of ones) across the 8 channels of a group; the slots
+//             are laid out as [g0 0..15][g0 16..N][g1 16..N][g1 0..15];
 //   warp 1    one thread issues tcgen05.mma (kind::f16, FP32 accumulate in
 //             TMEM): per group D1 = A(slots 0..15) x B(slots 0..N)^T, and
 //             for N >= 16 one D2 = A x B^T over the two groups' slots
-//             16..N together (the layout puts them side by side), so the
-//             extra rows cost one MMA instead of two half-empty ones; the
+//             16..N together (the layout puts them side by side); the
 //             useful entries of D are those with equal channel and group;
 //   warps 8-11 read TMEM (tcgen05.ld), keep each row's own-channel entries,
 //             and write the packed correlation (and optionally the sums).
-// Every wait is bounded (~2 s on the global timer); on expiry the kernel
-// records an error word, drains its in-flight copies and MMAs (again
-// bounded), frees its TMEM and returns.
+// Every wait is bounded by the plan's limit; on expiry the kernel records an
+// error word, drains its in-flight copies and MMAs (again bounded), frees its
+// TMEM and returns.
 //
 // gram_tc_f32_kernel (below) runs the same pipeline on float32 samples,
 // split into bf16 high and low parts on the way into shared memory.
@@ -50,18 +42,10 @@ namespace {
 constexpr int kBoxCh = 16;             // channels per TMA box (16 bytes)
 constexpr int kGroupSlots = 24;        // slots of an 8-channel group at most (N + 1 <= 24)
 constexpr int kMaxNU = 16;             // u8 ring depth bound (sized at launch)
-constexpr int kMaxNF = 4;              // f16 ring depth bound
+constexpr int kNF = 2;                 // f16 stages
 constexpr size_t kSmemBudget = 227 * 1024;
-
-// Tile shape of one kernel variant: T samples per stage, NF f16 stages.
-template <int T_, int NF_, int U_ = 1>
-struct TcCfg {
-  static constexpr int kT = T_;
-  static constexpr int kNF = NF_;
-  static constexpr int kUnroll = U_;  // converter loop unrolling
-  static constexpr int kSlotBytes = kT * 16;  // one slot: kT samples x 8 channels x f16
-  static_assert(kT % 16 == 0 && NF_ <= kMaxNF, "bad variant");
-};
+constexpr int kT = 64;                 // samples per stage
+constexpr int kSlotBytes = kT * 16;    // one slot: kT samples x 8 channels x f16
 constexpr int kThreads = 384;
 constexpr int kConvThreads = 128;
 constexpr int kEpiThreads = 128;
@@ -69,15 +53,12 @@ constexpr uint32_t kTmemCols = 512;
 
 struct TcArgs {
   int n_beam, n_chan, n_samp_sub, sub0, n_sub;
-  int n_pol;   // 2: blocks b and N + b are two polarisations of beam b, summed
-  int center;  // subtracted before f16: 128 (one polarisation), 255 (sum of two)
   int piece_stages;  // stages per TMEM accumulation; the epilogue adds the pieces
   int n_u8;  // u8 ring depth (stages), fixed at launch with the shared-memory size
   int R;    // slots per group: N + 1
   int R2;   // slots 16..N per group (0 if N + 1 <= 16)
   int rb;   // slots in B of the first MMAs (R rounded up to even)
   int64_t* sums;
-  int64_t* sums8;  // the same sums as [cell / 8][P][cell % 8] (internal layout)
   float* corr;
   unsigned long long* degenerate;
   unsigned* error;
@@ -109,7 +90,7 @@ __device__ __forceinline__ int d1_slot(int grp, int j, int R2) {
 
 struct Smem {
   uint64_t u8_full[kMaxNU], u8_empty[kMaxNU];
-  uint64_t f16_full[kMaxNF], f16_empty[kMaxNF];
+  uint64_t f16_full[kNF], f16_empty[kNF];
   uint64_t acc_full, acc_empty, drain;
   int epi_go;  // the epilogue leader's wait outcome
   uint32_t tmem_base;
@@ -123,44 +104,35 @@ struct Smem {
 __host__ __device__ constexpr int stage_slots(int n_beam) {
   return (2 * (n_beam + 1) + ((n_beam + 1) & 1)) > 32 ? (2 * (n_beam + 1) + ((n_beam + 1) & 1)) : 32;
 }
-template <class C>
 __host__ __device__ constexpr size_t f16_stage_bytes(int n_beam) {
-  return (size_t)stage_slots(n_beam) * C::kSlotBytes;
+  return (size_t)stage_slots(n_beam) * kSlotBytes;
 }
-// u8 ring depth for n_beam beams (n_pol blocks each): as deep as the
-// shared memory allows, so TMA keeps streaming while the MMAs pause for an
-// epilogue
-template <class C>
-__host__ __device__ constexpr int u8_ring_depth(int n_beam, int n_pol = 1) {
-  return (int)((kSmemBudget - 1024 - (size_t)C::kNF * f16_stage_bytes<C>(n_beam) - sizeof(Smem)) /
-               ((size_t)n_pol * n_beam * C::kT * kBoxCh)) < kMaxNU
-             ? (int)((kSmemBudget - 1024 - (size_t)C::kNF * f16_stage_bytes<C>(n_beam) -
-                      sizeof(Smem)) /
-                     ((size_t)n_pol * n_beam * C::kT * kBoxCh))
-             : kMaxNU;
+// bytes of one u8 stage: both polarisation blocks of n_beam beams
+__host__ __device__ constexpr size_t u8_stage_size(int n_beam) {
+  return (size_t)2 * n_beam * kT * kBoxCh;
+}
+// u8 ring depth: as deep as the shared memory allows, so TMA keeps streaming
+// while the MMAs pause for an epilogue
+__host__ __device__ constexpr int u8_ring_depth(int n_beam) {
+  const size_t room = kSmemBudget - 1024 - kNF * f16_stage_bytes(n_beam) - sizeof(Smem);
+  return (int)(room / u8_stage_size(n_beam)) < kMaxNU ? (int)(room / u8_stage_size(n_beam)) : kMaxNU;
 }
 // dynamic shared memory for n_beam beams and a ring of n_u8 stages
-template <class C>
-__host__ __device__ constexpr size_t smem_bytes(int n_beam, int n_u8, int n_pol = 1) {
-  return 1024 /* alignment slack */ + (size_t)C::kNF * f16_stage_bytes<C>(n_beam) +
-         (size_t)n_u8 * n_pol * n_beam * C::kT * kBoxCh + sizeof(Smem);
+__host__ __device__ constexpr size_t smem_bytes(int n_beam, int n_u8) {
+  return 1024 /* alignment slack */ + kNF * f16_stage_bytes(n_beam) +
+         (size_t)n_u8 * u8_stage_size(n_beam) + sizeof(Smem);
 }
 
-// kPol 2: the two-polarisation mode (converter adds blocks b and N + b;
-// the epilogue adds the TMEM pieces of a sub-integration as integers)
-template <int T_, int NF_, int U_, int kPol>
 __global__ void __launch_bounds__(kThreads, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
-  using C = TcCfg<T_, NF_, U_>;
-  constexpr int kT = C::kT, kNF = C::kNF, kSlotBytes = C::kSlotBytes;
-  const int kF16StageBytes = (int)f16_stage_bytes<C>(g.n_beam);
+  const int kF16StageBytes = (int)f16_stage_bytes(g.n_beam);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int kNU = g.n_u8;
   unsigned char* f16 = base;                                   // kNF stages
   unsigned char* u8 = f16 + (size_t)kNF * kF16StageBytes;      // kNU stages
-  const int u8_stage_bytes = g.n_pol * g.n_beam * kT * kBoxCh;
+  const int u8_stage_bytes = (int)u8_stage_size(g.n_beam);
   Smem* s = reinterpret_cast<Smem*>(u8 + (size_t)kNU * u8_stage_bytes);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -250,11 +222,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
       for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
         for (int st = 0; st < stages && ok; ++st, ++fcnt) {
           const int fs = fcnt % kNF;
-          // stage within the TMEM accumulation piece (the whole item for one
-          // polarisation)
-          int ps = st;
-          if constexpr (kPol == 2) ps = st % g.piece_stages;
-          const int last = kPol == 2 ? g.piece_stages - 1 : stages - 1;
+          const int ps = st % g.piece_stages;  // stage within the TMEM accumulation piece
+          const int last = g.piece_stages - 1;
           ok = mbar_wait(&s->f16_full[fs], (fcnt / kNF) & 1, g.error, g.wait_ns);
           if (!ok) break;
           if (ps == 0 && pcnt > 0) {
@@ -288,9 +257,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
   } else if (warp >= 4 && warp < 8) {
     // ------------------------------------------------------------ convert
     const int ct = threadIdx.x - 4 * 32;
-    const uint32_t magic = 0x64646464u;   // f16 bit pattern 0x64xx = 1024 + x
-    const uint32_t bias = 0x64806480u;    // f16x2 (1152, 1152)
-    const uint32_t bias2 = 0x64ff64ffu;   // f16x2 (1279, 1279): two polarisations
+    const uint32_t bias2 = 0x64ff64ffu;   // f16x2 (1279, 1279)
     uint32_t cnt = 0;
     bool ok = true;
     for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
@@ -301,49 +268,27 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
         if (!ok) break;
         const uint4* src = reinterpret_cast<const uint4*>(u8 + (size_t)us * u8_stage_bytes);
         unsigned char* dst = f16 + (size_t)fs * kF16StageBytes;
-        if constexpr (kPol == 2) {
-          // total power of two polarisations: x = p0 + p1 (0..510) in
-          // 16-bit lanes; f16 0x6400 | x = 1024 + x, minus 1279 gives
-          // x - 255 exactly (|x - 255| <= 255)
-          for (int r = ct; r < N * kT; r += kConvThreads) {
-            const uint4 wa = src[r], wb = src[r + N * kT];
-            const int b = r / kT, t = r % kT;
-            const uint32_t off = (t / 8) * 128 + (t % 8) * 16;
-            const uint32_t off0 = (uint32_t)b * kSlotBytes + off;
-            const uint32_t off1 = (uint32_t)slot_pos(1, b, g.R, g.R2) * kSlotBytes + off;
-            auto two = [&](uint32_t x, uint32_t y, uint32_t sel) {
-              const uint32_t v = (__byte_perm(x, 0u, sel) + __byte_perm(y, 0u, sel)) | 0x64006400u;
-              uint32_t o;
-              asm("sub.f16x2 %0, %1, %2;" : "=r"(o) : "r"(v), "r"(bias2));
-              return o;
-            };
-            const uint4 o0 = make_uint4(two(wa.x, wb.x, 0x4140), two(wa.x, wb.x, 0x4342),
-                                        two(wa.y, wb.y, 0x4140), two(wa.y, wb.y, 0x4342));
-            const uint4 o1 = make_uint4(two(wa.z, wb.z, 0x4140), two(wa.z, wb.z, 0x4342),
-                                        two(wa.w, wb.w, 0x4140), two(wa.w, wb.w, 0x4342));
-            *reinterpret_cast<uint4*>(dst + off0) = o0;
-            *reinterpret_cast<uint4*>(dst + off1) = o1;
-          }
-        } else {
-#pragma unroll C::kUnroll
+        // total power of two polarisations: x = p0 + p1 (0..510) in
+        // 16-bit lanes; f16 0x6400 | x = 1024 + x, minus 1279 gives
+        // x - 255 exactly (|x - 255| <= 255)
         for (int r = ct; r < N * kT; r += kConvThreads) {
-          const uint4 w = src[r];  // 16 channels of beam b at sample t
+          const uint4 wa = src[r], wb = src[r + N * kT];
           const int b = r / kT, t = r % kT;
           const uint32_t off = (t / 8) * 128 + (t % 8) * 16;
           const uint32_t off0 = (uint32_t)b * kSlotBytes + off;
           const uint32_t off1 = (uint32_t)slot_pos(1, b, g.R, g.R2) * kSlotBytes + off;
-          uint4 o0, o1;
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o0.x) : "r"(__byte_perm(w.x, magic, 0x4140)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o0.y) : "r"(__byte_perm(w.x, magic, 0x4342)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o0.z) : "r"(__byte_perm(w.y, magic, 0x4140)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o0.w) : "r"(__byte_perm(w.y, magic, 0x4342)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o1.x) : "r"(__byte_perm(w.z, magic, 0x4140)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o1.y) : "r"(__byte_perm(w.z, magic, 0x4342)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o1.z) : "r"(__byte_perm(w.w, magic, 0x4140)), "r"(bias));
-          asm("sub.f16x2 %0, %1, %2;" : "=r"(o1.w) : "r"(__byte_perm(w.w, magic, 0x4342)), "r"(bias));
+          auto two = [&](uint32_t x, uint32_t y, uint32_t sel) {
+            const uint32_t v = (__byte_perm(x, 0u, sel) + __byte_perm(y, 0u, sel)) | 0x64006400u;
+            uint32_t o;
+            asm("sub.f16x2 %0, %1, %2;" : "=r"(o) : "r"(v), "r"(bias2));
+            return o;
+          };
+          const uint4 o0 = make_uint4(two(wa.x, wb.x, 0x4140), two(wa.x, wb.x, 0x4342),
+                                      two(wa.y, wb.y, 0x4140), two(wa.y, wb.y, 0x4342));
+          const uint4 o1 = make_uint4(two(wa.z, wb.z, 0x4140), two(wa.z, wb.z, 0x4342),
+                                      two(wa.w, wb.w, 0x4140), two(wa.w, wb.w, 0x4342));
           *reinterpret_cast<uint4*>(dst + off0) = o0;
           *reinterpret_cast<uint4*>(dst + off1) = o1;
-        }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(&s->u8_empty[us]);
@@ -366,8 +311,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
     bool ok = true;
     for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
       // the rest of the item from the rows D1 `slot` of each group and D2
-      // `slot2` (by column block): floats of exact integers (one
-      // polarisation) or int32 sums of the pieces (two)
+      // `slot2` (by column block): int32 sums of the pieces
       auto finish = [&](auto& row, auto& row2) {
         // G[a][N] (row sum) and G[a][a] from each row, picked with
         // compile-time register indices and runtime block -> slot maps
@@ -437,27 +381,22 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
               dst[b - a] = r;
             }
           }
-          if (g.sums || g.sums8) {
+          if (g.sums) {
             const int N1 = N + 1;
             const int64_t P = N1 * (N1 + 1) / 2;
             const int row = a * N1 - a * (a - 1) / 2;
-            // public layout: one cell's entries contiguous; interleaved: the
-            // 8 channels of a group side by side, so a warp's 8-byte stores
-            // fill 64-byte runs
-            int64_t* dst = g.sums8 ? g.sums8 + ((cell >> 3) * P + row) * 8 + (cell & 7)
-                                   : g.sums + cell * P + row;
-            const int step = g.sums8 ? 8 : 1;
+            int64_t* dst = g.sums + cell * P + row;
   #pragma unroll
             for (int jb = 0; jb < NB; ++jb) {
               const int b = slot_of(jb);
               if (b < a || b > N) continue;
               const int64_t gab = (int64_t)rv[jb];
               int64_t v;
-              const int64_t cc = g.center;
+              const int64_t cc = 255;  // the converter's centre
               if (a == N) v = n;                                  // (N, N): sample count
               else if (b == N) v = gab + cc * n;                  // S_a
               else v = gab + cc * (sa + (int64_t)s->s_sum[grp][c][b]) + cc * cc * n;
-              dst[(b - a) * step] = v;
+              dst[b - a] = v;
             }
           }
         };
@@ -471,46 +410,6 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
                [&](int jb) { return (jb >= jb2 && jb < jb2 + R2) ? 16 + jb - jb2 : -1; });
         named_sync(1, kEpiThreads);  // smem tables reused by the next item
       };
-      if constexpr (kPol == 1) {
-        ok = epi_wait(&s->acc_full, pcnt & 1, g.error, g.wait_ns, &s->epi_go,
-                      threadIdx.x == 256);
-        if (!ok) break;
-        ++pcnt;
-        fence_after();
-        float row[2][kGroupSlots];   // D1 row `slot` of each group, by column block
-        float row2[16];              // D2 row `slot2`, by column block
-#pragma unroll
-        for (int grp = 0; grp < 2; ++grp) {
-          // chunks of 32 columns (4 blocks x 8 channels), one load in flight
-#pragma unroll
-          for (int ch = 0; ch < kGroupSlots / 4; ++ch) {
-            if (ch * 4 < g.rb) {
-              uint32_t v[32];
-              tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + grp * 192 + ch * 32, v);
-              tmem_wait_ld();
-              pick4(v, c, &row[grp][4 * ch]);
-            } else {
-#pragma unroll
-              for (int u = 0; u < 4; ++u) row[grp][4 * ch + u] = 0.f;
-            }
-          }
-        }
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          if (2 * R2 > 4 * ch) {
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + 384 + ch * 32, v);
-            tmem_wait_ld();
-            pick4(v, c, &row2[4 * ch]);
-          } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) row2[4 * ch + u] = 0.f;
-          }
-        }
-        fence_before();
-        mbar_arrive(&s->acc_empty);  // accumulators may be overwritten now
-        finish(row, row2);
-      } else {
         // exact integer sums over the accumulation pieces (each piece's
         // sums are integers below 2^24, so exact in FP32; the total fits int32)
         const int pieces = stages / g.piece_stages;
@@ -559,538 +458,6 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
         }
         if (!ok) break;
         finish(row, row2);
-      }
-    }
-  }
-  __syncthreads();
-  if (warp == 2) {
-    fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(kTmemCols));
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The same Gram with the A operand in tensor memory (variants 8 and 9; one
-// polarisation, N + 1 <= 20 slots). In the kernel above the tensor core
-// reads A (16 beam slots x 8 channels) and B from shared memory: about 96 B
-// of operand reads per channel-sample, which with the TMA writes and the
-// converter's traffic keeps the SM's shared-memory path ~80 % busy at half
-// of HBM. Here the converter writes A straight into TMEM. ldmatrix .trans
-// .b8 turns a 16-sample x 16-channel byte tile of one beam into 4
-// consecutive samples of channel p and of channel p + 8 per lane (p = lane
-// / 4, samples 4 (lane % 4) ..); two beams' registers (slots s, s + 1) fill
-// one tcgen05.st 16x256b store, i.e. 16 TMEM lanes (8 channels x 2 slots,
-// lane = 8 slot + channel) by 16 K values, which is the K-major A layout of
-// kind::f16. The same registers give B in the K-major canonical layout
-// (8-byte stores, a warp's 256 contiguous bytes). Only B is read from
-// shared memory by the MMA, half the operand bytes. Operands go through
-// sub-stages of 16 samples (one K step each): B in shared memory, A in TMEM
-// columns after the accumulators (D1 of group 0 at column 0, of group 1 at
-// 8 rb, D2 at 16 rb; 24 columns per sub-stage for A of group 0, group 1 and
-// D2), as many sub-stages as the 512 columns leave (5 for 19 beams).
-constexpr int kMaxNA = 8;  // A/B sub-stages bound
-constexpr int kASub = 16;  // samples per A/B sub-stage (one K step)
-
-__host__ __device__ constexpr int tca_g1_col(int rb) { return 8 * rb; }
-__host__ __device__ constexpr int tca_d2_col(int rb) { return 16 * rb; }
-__host__ __device__ constexpr int tca_a_col(int rb, int R2) { return 16 * rb + 16 * R2; }
-__host__ __device__ constexpr int tca_sub_stages(int rb, int R2) {
-  return ((int)kTmemCols - tca_a_col(rb, R2)) / 24 < kMaxNA
-             ? ((int)kTmemCols - tca_a_col(rb, R2)) / 24
-             : kMaxNA;
-}
-// bytes of one B sub-stage: every slot of both groups, 16 samples x 8 channels x f16
-__host__ __device__ constexpr int tca_sub_bytes(int n_beam) { return stage_slots(n_beam) * 256; }
-
-struct SmemA {
-  uint64_t u8_full[kMaxNU], u8_empty[kMaxNU];
-  uint64_t f16_full[kMaxNA], f16_empty[kMaxNA];
-  uint64_t acc_full, acc_empty, drain;
-  int epi_go;  // the epilogue leader's wait outcome
-  uint32_t tmem_base;
-  int32_t s_sum[2][8][kGroupSlots];
-  float s_inv[2][8][kGroupSlots];
-};
-template <int T_>
-__host__ __device__ constexpr int tca_u8_depth(int n_beam, int na) {
-  return (int)((kSmemBudget - 1024 - (size_t)na * tca_sub_bytes(n_beam) - sizeof(SmemA)) /
-               ((size_t)n_beam * T_ * kBoxCh)) < kMaxNU
-             ? (int)((kSmemBudget - 1024 - (size_t)na * tca_sub_bytes(n_beam) - sizeof(SmemA)) /
-                     ((size_t)n_beam * T_ * kBoxCh))
-             : kMaxNU;
-}
-template <int T_>
-__host__ __device__ constexpr size_t tca_smem_bytes(int n_beam, int na, int n_u8) {
-  return 1024 + (size_t)na * tca_sub_bytes(n_beam) + (size_t)n_u8 * n_beam * T_ * kBoxCh +
-         sizeof(SmemA);
-}
-__device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b,
-                                           uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate));
-}
-__device__ __forceinline__ void tmem_st16x256(uint32_t taddr, uint32_t v0, uint32_t v1, uint32_t v2,
-                                              uint32_t v3) {
-  asm volatile("tcgen05.st.sync.aligned.16x256b.x1.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr),
-               "r"(v0), "r"(v1), "r"(v2), "r"(v3)
-               : "memory");
-}
-template <int T_>
-__global__ void __launch_bounds__(kThreads, 1)
-gram_tc_a_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
-  constexpr int kT = T_, kPol = 1;
-  const int kNA = tca_sub_stages(g.rb, g.R2);
-  const int kSubBytes = tca_sub_bytes(g.n_beam);
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  unsigned char* base =
-      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int kNU = g.n_u8;
-  unsigned char* f16 = base;                                   // kNA B sub-stages
-  unsigned char* u8 = f16 + (size_t)kNA * kSubBytes;           // kNU stages
-  const int u8_stage_bytes = g.n_beam * kT * kBoxCh;
-  SmemA* s = reinterpret_cast<SmemA*>(u8 + (size_t)kNU * u8_stage_bytes);
-
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int N = g.n_beam;
-  const int chunks = g.n_chan / kBoxCh;
-  const int64_t items = (int64_t)g.n_sub * chunks;
-  const int stages = g.n_samp_sub / kT;
-  const int g1c = tca_g1_col(g.rb), d2c = tca_d2_col(g.rb), ac = tca_a_col(g.rb, g.R2);
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kNU; ++i) {
-      mbar_init(&s->u8_full[i], 1);
-      mbar_init(&s->u8_empty[i], kConvThreads);
-    }
-    for (int i = 0; i < kNA; ++i) {
-      mbar_init(&s->f16_full[i], kConvThreads);
-      mbar_init(&s->f16_empty[i], 1);
-    }
-    mbar_init(&s->acc_full, 1);
-    mbar_init(&s->acc_empty, kEpiThreads);
-    mbar_init(&s->drain, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  // B sub-stages: the rows of ones (slot N of each group) and zeros where
-  // the converter does not write (slots past N)
-  const uint32_t one2 = 0x3c003c00u;  // f16x2 (1.0, 1.0)
-  const int p_one0 = slot_pos(0, N, g.R, g.R2), p_one1 = slot_pos(1, N, g.R, g.R2);
-  for (int st = 0; st < kNA; ++st) {
-    uint32_t* w = reinterpret_cast<uint32_t*>(f16 + (size_t)st * kSubBytes);
-    for (int i = threadIdx.x; i < kSubBytes / 4; i += blockDim.x) {
-      const int pos = i / 64;  // 256 B per slot
-      w[i] = (pos == p_one0 || pos == p_one1) ? one2 : 0u;
-    }
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  if (warp == 2) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(&s->tmem_base)),
-                 "r"(kTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  __syncthreads();
-  fence_after();
-  const uint32_t tmem = s->tmem_base;
-
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA
-    if (lane == 0) {
-      uint32_t cnt = 0;
-      long long withheld = -1;
-      bool ok = true;
-      for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const int k = (int)(it / chunks), ch0 = (int)(it % chunks) * kBoxCh;
-        const int64_t t_item = (int64_t)(g.sub0 + k) * g.n_samp_sub;
-        for (int st = 0; st < stages && ok; ++st, ++cnt) {
-          const int slot = cnt % kNU;
-          ok = mbar_wait(&s->u8_empty[slot], ((cnt / kNU) & 1) ^ 1, g.error, g.wait_ns);
-          if (!ok) break;
-          if (blockIdx.x == 0 && (long long)cnt == g.withhold) {
-            // injected fault: this stage is never issued, so the converter's
-            // bounded wait for it expires (nothing is in flight for it)
-            withheld = cnt;
-            continue;
-          }
-          mbar_expect_tx(&s->u8_full[slot], (uint32_t)u8_stage_bytes);
-          tma_load_3d(u8 + (size_t)slot * u8_stage_bytes, &tmap, ch0, (int)(t_item + st * kT), 0,
-                      &s->u8_full[slot]);
-        }
-      }
-      // drain: every issued copy has landed before the CTA may exit
-      for (uint32_t d = cnt > kNU ? cnt - kNU : 0; d < cnt; ++d)
-        if ((long long)d != withheld)
-          mbar_drain(&s->u8_full[d % kNU], (d / kNU) & 1, g.error, g.wait_ns);
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA
-    if (lane == 0) {
-      const uint32_t f16_base = smem_u32(f16);
-      const uint32_t id1 = idesc_f16_k(128, 8 * g.rb);
-      const uint32_t id2 = idesc_f16_k(128, g.R2 > 0 ? 16 * g.R2 : 16);
-      const uint32_t pb1 = (uint32_t)g.R * 256;  // group 1's B: positions R ..
-      const uint32_t pb2 = 16u * 256;            // D2's B: positions 16 ..
-      // K-major canonical layout, no swizzle: core matrices of 8 rows x 16 B,
-      // K-adjacent ones 128 B apart, the next 8 rows (slot) 256 B on
-      const uint32_t lbo = 128, sbo = 256;
-      const int subs = stages * (kT / kASub);
-      uint32_t fcnt = 0, pcnt = 0;
-      bool ok = true;
-      for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        for (int st = 0; st < subs && ok; ++st, ++fcnt) {
-          const int fs = fcnt % kNA;
-          ok = mbar_wait(&s->f16_full[fs], (fcnt / kNA) & 1, g.error, g.wait_ns);
-          if (!ok) break;
-          if (st == 0 && pcnt > 0) {
-            ok = mbar_wait(&s->acc_empty, (pcnt - 1) & 1, g.error, g.wait_ns);
-            if (!ok) break;
-          }
-          fence_after();
-          const uint32_t b = f16_base + (uint32_t)(fs * kSubBytes);
-          const uint32_t a = tmem + (uint32_t)(ac + 24 * fs);
-          const uint32_t acc = st > 0 ? 1u : 0u;
-          mma_f16_ta(tmem, a, smem_desc(b, lbo, sbo), id1, acc);
-          mma_f16_ta(tmem + g1c, a + 8, smem_desc(b + pb1, lbo, sbo), id1, acc);
-          if (g.R2 > 0) mma_f16_ta(tmem + d2c, a + 16, smem_desc(b + pb2, lbo, sbo), id2, acc);
-          mma_commit(&s->f16_empty[fs]);  // sub-stage free once these MMAs finish
-          if (st == subs - 1) {
-            mma_commit(&s->acc_full);
-            ++pcnt;
-          }
-        }
-      }
-      mma_commit(&s->drain);  // every MMA issued has finished before TMEM is freed
-      mbar_drain(&s->drain, 0, g.error, g.wait_ns);
-    }
-  } else if (warp >= 4 && warp < 8) {
-    // ------------------------------------------------------------ convert
-    // Warp w4 = warp - 4 writes TMEM lanes 32 w4 .. 32 w4 + 31: the A rows of
-    // slots 4 w4 .. 4 w4 + 3 for both groups, and of D2 positions 4 w4 ..
-    // 4 w4 + 3; it writes the B rows of the beams it loads.
-    const int w4 = warp - 4;
-    const int p = lane / 4, q = lane % 4;
-    const uint32_t u8_base = smem_u32(u8);
-    const uint32_t f16_base_c = smem_u32(f16);
-    // this lane's 8 bytes in a slot's 16 samples: K block q / 2, row p
-    const uint32_t bq = (uint32_t)((q / 2) * 128 + p * 16 + (q % 2) * 8);
-    const int ksub = kT / kASub;
-    // The slots this warp converts, fixed for the launch: entries 0..3 are
-    // D1 slots 4 w4 + k (both groups), entries 4..7 D2 positions 2u + h for
-    // u = 2 w4 + j (j = 0, 1), of group grp. kind 0: a beam (loaded), 1: the
-    // row of ones, 2: zeros (or nothing to write). src: the ldmatrix row
-    // address of this lane in the slot's u8 tile; b0 / b1: this lane's B
-    // bytes in a sub-stage for group 0 / 1 (entries 4..7: of their group).
-    int kind[8], grp2[4];
-    uint32_t src[8], b0[8], b1[4];
-    bool d2_on[2];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      int slot, grp = 0;
-      bool on = true;
-      if (k < 4) {
-        slot = 4 * w4 + k;
-      } else {
-        const int j = (k - 4) / 2, h = (k - 4) % 2, u = 2 * w4 + j;
-        on = u < g.R2;
-        if (h == 0) d2_on[j] = on;
-        const int i = 2 * u + h;
-        grp = i < g.R2 ? 0 : 1;
-        slot = 16 + (grp ? i - g.R2 : i);
-        grp2[k - 4] = grp;
-      }
-      kind[k] = !on ? 2 : (slot < N ? 0 : (slot == N ? 1 : 2));
-      src[k] = (uint32_t)((slot < N ? slot : 0) * kT * kBoxCh + (lane & 15) * kBoxCh);
-      b0[k] = (uint32_t)slot_pos(grp, slot, g.R, g.R2) * 256 + bq;
-      if (k < 4) b1[k] = (uint32_t)slot_pos(1, slot, g.R, g.R2) * 256 + bq;
-    }
-    auto st_b = [&](uint32_t addr, uint32_t x, uint32_t y) {
-      asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
-    };
-    uint32_t cnt = 0, fcnt = 0;
-    bool ok = true;
-    for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
-      for (int st = 0; st < stages && ok; ++st, ++cnt) {
-        const int us = cnt % kNU;
-        ok = mbar_wait(&s->u8_full[us], (cnt / kNU) & 1, g.error, g.wait_ns);
-        if (!ok) break;
-        const uint32_t u8_stage = u8_base + (uint32_t)us * (uint32_t)u8_stage_bytes;
-        for (int ks = 0; ks < ksub && ok; ++ks, ++fcnt) {
-          const int fs = fcnt % kNA;
-          ok = mbar_wait(&s->f16_empty[fs], ((fcnt / kNA) & 1) ^ 1, g.error, g.wait_ns);
-          if (!ok) break;
-          fence_after();  // the MMAs that read this sub-stage's A columns have finished
-          const uint32_t bsub = f16_base_c + (uint32_t)(fs * kSubBytes);
-          const uint32_t acol = tmem + ((uint32_t)(32 * w4) << 16) + (uint32_t)(ac + 24 * fs);
-          const uint32_t rows = u8_stage + (uint32_t)(ks * kASub * kBoxCh);
-          // every load first (one latency for all), then the conversions,
-          // then the B and A stores. Thread (p, q) gets samples 4q..4q+3 of
-          // channels p and p + 8: f16x2 registers v[k][0..1] and v[k][2..3].
-          uint32_t raw[8][2], v[8][4];
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            if (kind[k] == 0) ldm_trans_b8(rows + src[k], raw[k][0], raw[k][1]);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            if (kind[k] == 0) {
-              u8x4_to_f16(raw[k][0], v[k][0], v[k][1]);
-              u8x4_to_f16(raw[k][1], v[k][2], v[k][3]);
-            } else {
-              const uint32_t c1 = kind[k] == 1 ? one2 : 0u;
-              v[k][0] = v[k][1] = v[k][2] = v[k][3] = c1;
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (kind[k] == 0) {
-              st_b(bsub + b0[k], v[k][0], v[k][1]);
-              st_b(bsub + b1[k], v[k][2], v[k][3]);
-            }
-#pragma unroll
-          for (int k = 4; k < 8; ++k)
-            if (kind[k] == 0) {
-              const bool g1 = grp2[k - 4] != 0;
-              st_b(bsub + b0[k], g1 ? v[k][2] : v[k][0], g1 ? v[k][3] : v[k][1]);
-            }
-          // D1 A: slots 4 w4 + 2j, + 1 -> lanes 32 w4 + 16 j ..; group 1 eight columns on
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const uint32_t lanes = (uint32_t)(16 * j) << 16;
-            const int k = 2 * j;
-            tmem_st16x256(acol + lanes, v[k][0], v[k][1], v[k + 1][0], v[k + 1][1]);
-            tmem_st16x256(acol + lanes + 8, v[k][2], v[k][3], v[k + 1][2], v[k + 1][3]);
-          }
-          // D2 A: positions 2u, 2u + 1 -> lanes 16 u .., sixteen columns on
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            if (!d2_on[j]) continue;
-            const int k = 4 + 2 * j;
-            const bool ga = grp2[2 * j] != 0, gb = grp2[2 * j + 1] != 0;
-            tmem_st16x256(acol + ((uint32_t)(16 * j) << 16) + 16, ga ? v[k][2] : v[k][0],
-                          ga ? v[k][3] : v[k][1], gb ? v[k + 1][2] : v[k + 1][0],
-                          gb ? v[k + 1][3] : v[k + 1][1]);
-          }
-          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          fence_before();
-          mbar_arrive(&s->f16_full[fs]);
-        }
-        if (!ok) break;
-        mbar_arrive(&s->u8_empty[us]);
-      }
-    }
-  } else if (warp >= 8) {
-    // ------------------------------------------------------------ epilogue
-    const int q = warp - 8;              // TMEM lane quarter (warp % 4)
-    const int c = lane % 8;              // channel within the group
-    const int slot = 4 * q + lane / 8;   // D1 row slot (beam a, 0..15), both groups
-    // D2 row of this lane: stage position 16 + 4q + lane/8, which holds
-    // slot 16.. of group 0, then slot 16.. of group 1, then nothing useful
-    const int p2 = 4 * q + lane / 8;     // position - 16
-    const int g2 = p2 < g.R2 ? 0 : (p2 < 2 * g.R2 ? 1 : -1);
-    const int slot2 = 16 + (g2 == 1 ? p2 - g.R2 : p2);
-    const int64_t n = g.n_samp_sub;
-    const int R = g.R, R2 = g.R2;
-    uint32_t pcnt = 0;
-    bool ok = true;
-    for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
-      // the rest of the item from the rows D1 `slot` of each group and D2
-      // `slot2` (by column block): floats of exact integers (one
-      // polarisation) or int32 sums of the pieces (two)
-      auto finish = [&](auto& row, auto& row2) {
-        // G[a][N] (row sum) and G[a][a] from each row, picked with
-        // compile-time register indices and runtime block -> slot maps
-        using V = std::remove_reference_t<decltype(row[0][0])>;
-        V sumN[2], diag[2], sumN2 = 0, diag2 = 0;
-  #pragma unroll
-        for (int grp = 0; grp < 2; ++grp) {
-          sumN[grp] = diag[grp] = 0;
-  #pragma unroll
-          for (int jb = 0; jb < kGroupSlots; ++jb) {
-            const int b = d1_slot(grp, jb, R2);
-            if (jb < R && b == N) sumN[grp] = row[grp][jb];
-            if (jb < R && b == slot) diag[grp] = row[grp][jb];
-          }
-        }
-        // D2 columns: blocks 0..R2-1 are group 0 slots 16.., then group 1's
-        const int jb2 = g2 == 1 ? R2 : 0;
-  #pragma unroll
-        for (int jb = 0; jb < 16; ++jb) {
-          if (jb - jb2 == N - 16) sumN2 = row2[jb];
-          if (jb - jb2 == slot2 - 16) diag2 = row2[jb];
-        }
-
-        const int k = (int)(it / chunks), ch0 = (int)(it % chunks) * kBoxCh;
-        // row sums and inverse standard deviations, shared through smem
-        auto table = [&](int grp, int a, V sum_a, V diag_a) {
-          const int64_t sa = (int64_t)sum_a;
-          const int64_t var = n * (int64_t)diag_a - sa * sa;
-          s->s_sum[grp][c][a] = (int32_t)sa;
-          float inv = 0.f;
-          if (a < N) {
-            if (var > 0) {
-              const float vf = (float)var;
-              inv = rsqrtf(vf);
-              inv = inv * (1.5f - 0.5f * vf * inv * inv);
-            } else {
-              atomicAdd(g.degenerate, 1ull);
-            }
-          }
-          s->s_inv[grp][c][a] = inv;
-        };
-  #pragma unroll
-        for (int grp = 0; grp < 2; ++grp)
-          if (slot < N + 1) table(grp, slot, sumN[grp], diag[grp]);
-        if (g2 >= 0 && slot2 < N + 1) table(g2, slot2, sumN2, diag2);
-        named_sync(1, kEpiThreads);
-        // one packed output row: a, its group, its values by column block and
-        // the slot of each block (b < 0: not this group's)
-        auto emit = [&](int grp, int a, const V* rv, auto nb_c, auto slot_of) {
-          constexpr int NB = decltype(nb_c)::value;
-          const int64_t cell = (int64_t)k * g.n_chan + ch0 + grp * 8 + c;
-          const int64_t sa = s->s_sum[grp][c][a];
-          const float inva = s->s_inv[grp][c][a];
-          if (g.corr && a < N) {
-            float* dst = g.corr + cell * (int64_t)(N * (N + 1) / 2) + (a * N - a * (a - 1) / 2);
-  #pragma unroll
-            for (int jb = 0; jb < NB; ++jb) {
-              const int b = slot_of(jb);
-              if (b < a || b >= N) continue;
-              float r;
-              if (b == a) {
-                r = 1.f;
-              } else {
-                const int64_t cov = n * (int64_t)rv[jb] - sa * (int64_t)s->s_sum[grp][c][b];
-                r = (float)cov * inva * s->s_inv[grp][c][b];
-              }
-              dst[b - a] = r;
-            }
-          }
-          if (g.sums || g.sums8) {
-            const int N1 = N + 1;
-            const int64_t P = N1 * (N1 + 1) / 2;
-            const int row = a * N1 - a * (a - 1) / 2;
-            // public layout: one cell's entries contiguous; interleaved: the
-            // 8 channels of a group side by side, so a warp's 8-byte stores
-            // fill 64-byte runs
-            int64_t* dst = g.sums8 ? g.sums8 + ((cell >> 3) * P + row) * 8 + (cell & 7)
-                                   : g.sums + cell * P + row;
-            const int step = g.sums8 ? 8 : 1;
-  #pragma unroll
-            for (int jb = 0; jb < NB; ++jb) {
-              const int b = slot_of(jb);
-              if (b < a || b > N) continue;
-              const int64_t gab = (int64_t)rv[jb];
-              int64_t v;
-              const int64_t cc = g.center;
-              if (a == N) v = n;                                  // (N, N): sample count
-              else if (b == N) v = gab + cc * n;                  // S_a
-              else v = gab + cc * (sa + (int64_t)s->s_sum[grp][c][b]) + cc * cc * n;
-              dst[(b - a) * step] = v;
-            }
-          }
-        };
-  #pragma unroll
-        for (int grp = 0; grp < 2; ++grp)
-          if (slot <= N)
-            emit(grp, slot, row[grp], std::integral_constant<int, kGroupSlots>{},
-                 [&](int jb) { return jb < R ? d1_slot(grp, jb, R2) : -1; });
-        if (g2 >= 0 && slot2 <= N)
-          emit(g2, slot2, row2, std::integral_constant<int, 16>{},
-               [&](int jb) { return (jb >= jb2 && jb < jb2 + R2) ? 16 + jb - jb2 : -1; });
-        named_sync(1, kEpiThreads);  // smem tables reused by the next item
-      };
-      if constexpr (kPol == 1) {
-        ok = epi_wait(&s->acc_full, pcnt & 1, g.error, g.wait_ns, &s->epi_go,
-                      threadIdx.x == 256);
-        if (!ok) break;
-        ++pcnt;
-        fence_after();
-        float row[2][kGroupSlots];   // D1 row `slot` of each group, by column block
-        float row2[16];              // D2 row `slot2`, by column block
-#pragma unroll
-        for (int grp = 0; grp < 2; ++grp) {
-          // chunks of 32 columns (4 blocks x 8 channels), one load in flight
-#pragma unroll
-          for (int ch = 0; ch < kGroupSlots / 4; ++ch) {
-            if (ch * 4 < g.rb) {
-              uint32_t v[32];
-              tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + grp * g1c + ch * 32, v);
-              tmem_wait_ld();
-              pick4(v, c, &row[grp][4 * ch]);
-            } else {
-#pragma unroll
-              for (int u = 0; u < 4; ++u) row[grp][4 * ch + u] = 0.f;
-            }
-          }
-        }
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          if (2 * R2 > 4 * ch) {
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + d2c + ch * 32, v);
-            tmem_wait_ld();
-            pick4(v, c, &row2[4 * ch]);
-          } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) row2[4 * ch + u] = 0.f;
-          }
-        }
-        fence_before();
-        mbar_arrive(&s->acc_empty);  // accumulators may be overwritten now
-        finish(row, row2);
-      } else {
-        // exact integer sums over the accumulation pieces (each piece's
-        // sums are integers below 2^24, so exact in FP32; the total fits int32)
-        const int pieces = stages / g.piece_stages;
-        int32_t row[2][kGroupSlots];
-        int32_t row2[16];
-#pragma unroll
-        for (int grp = 0; grp < 2; ++grp)
-#pragma unroll
-          for (int jb = 0; jb < kGroupSlots; ++jb) row[grp][jb] = 0;
-#pragma unroll
-        for (int jb = 0; jb < 16; ++jb) row2[jb] = 0;
-        for (int pc = 0; pc < pieces && ok; ++pc, ++pcnt) {
-          ok = epi_wait(&s->acc_full, pcnt & 1, g.error, g.wait_ns, &s->epi_go,
-                        threadIdx.x == 256);
-          if (!ok) break;
-          fence_after();
-#pragma unroll
-          for (int grp = 0; grp < 2; ++grp) {
-#pragma unroll
-            for (int ch = 0; ch < kGroupSlots / 4; ++ch) {
-              if (ch * 4 < g.rb) {
-                uint32_t v[32];
-                float f4[4];
-                tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + grp * g1c + ch * 32, v);
-                tmem_wait_ld();
-                pick4(v, c, f4);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) row[grp][4 * ch + u] += __float2int_rn(f4[u]);
-              }
-            }
-          }
-#pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            if (2 * R2 > 4 * ch) {
-              uint32_t v[32];
-              float f4[4];
-              tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + d2c + ch * 32, v);
-              tmem_wait_ld();
-              pick4(v, c, f4);
-#pragma unroll
-              for (int u = 0; u < 4; ++u) row2[4 * ch + u] += __float2int_rn(f4[u]);
-            }
-          }
-          fence_before();
-          mbar_arrive(&s->acc_empty);
-        }
-        if (!ok) break;
-        finish(row, row2);
-      }
     }
   }
   __syncthreads();
@@ -1472,79 +839,26 @@ gram_tc_f32_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
 
 }  // namespace
 
-// Tensor-core Gram variants {samples per stage, f16 stages, converter
-// unrolling}: 0 = {64, 2, 1}, 1 = {32, 4, 1}, 2 = {32, 2, 1}, 3 = {64, 3, 1},
-// 4 = {64, 2, 2}, 5 = {64, 3, 2}, 6 = {64, 4, 1}, 7 = {64, 4, 2}; with A in
-// TMEM (gram_tc_a_kernel, up to 19 beams): 8 = 64-sample TMA stages, 9 = 32.
-int tc_variant_samples(int v) { return (v == 1 || v == 2 || v == 9) ? 32 : 64; }
-
-// Untuned default: four f16 stages of 64 samples where that still leaves
-// an u8 ring of at least three stages (measured fastest for 19 beams),
-// else two.
-int tc_default_variant(int n_beam) {
-  if (n_beam < 2 || n_beam + 1 > kGroupSlots) return 0;
-  return u8_ring_depth<TcCfg<64, 4, 1>>(n_beam) >= 3 ? 6 : 0;
-}
-
-
-// u8 ring depth of variant v for n_beam beams of n_pol blocks
-static int tc_u8_depth(int v, int n_beam, int n_pol) {
-  switch (v) {
-    case 1: return u8_ring_depth<TcCfg<32, 4, 1>>(n_beam, n_pol);
-    case 2: return u8_ring_depth<TcCfg<32, 2, 1>>(n_beam, n_pol);
-    case 3: return u8_ring_depth<TcCfg<64, 3, 1>>(n_beam, n_pol);
-    case 4: return u8_ring_depth<TcCfg<64, 2, 2>>(n_beam, n_pol);
-    case 5: return u8_ring_depth<TcCfg<64, 3, 2>>(n_beam, n_pol);
-    case 6: return u8_ring_depth<TcCfg<64, 4, 1>>(n_beam, n_pol);
-    case 7: return u8_ring_depth<TcCfg<64, 4, 2>>(n_beam, n_pol);
-    default: return u8_ring_depth<TcCfg<64, 2, 1>>(n_beam, n_pol);
-  }
-}
-
-// The A-in-TMEM kernel fits where the accumulators leave TMEM room for at
-// least two operand sub-stages and shared memory an u8 ring of two stages.
-static bool tca_fits(int v, int n_beam) {
-  const int R = n_beam + 1, rb = (R + 1) / 2 * 2, R2 = R > 16 ? R - 16 : 0;
-  if (n_beam < 2 || R > 20 || tca_sub_stages(rb, R2) < 2) return false;
-  const int na = tca_sub_stages(rb, R2);
-  return (v == 9 ? tca_u8_depth<32>(n_beam, na) : tca_u8_depth<64>(n_beam, na)) >= 2;
-}
-
-// Two polarisations double the u8 stage: they run variant 0 (two f16
-// stages), which leaves the u8 ring at least two stages deep. Variants 8
-// and 9 where they do not fit the shape run the untuned default.
-static int tc_variant_for(const mraid_plan_s* pl, int n_pol) {
-  if (n_pol == 2) return 0;
-  const int v = pl->tc_variant;
-  if (v >= 8 && !tca_fits(v, pl->p.n_beam)) return tc_default_variant(pl->p.n_beam);
-  return v;
-}
-
-int tc_variant_effective(const mraid_plan_s* pl) { return tc_variant_for(pl, 1); }
-
-bool gram_tc_supported(const mraid_plan_s* pl, const void* d_data, int n_pol) {
+bool gram_tc_pol2_supported(const mraid_plan_s* pl, const void* d_data) {
   const mraid_params& p = pl->p;
-  const int t = tc_variant_samples(tc_variant_for(pl, n_pol));
   return p.bit_depth == 8 && p.n_beam >= 2 && p.n_beam + 1 <= kGroupSlots &&
-         (n_pol == 1 || (n_pol == 2 && tc_u8_depth(tc_variant_for(pl, 2), p.n_beam, 2) >= 2)) &&
-         p.n_samp_sub % t == 0 && p.n_samp_sub <= 1024 && p.n_chan % kBoxCh == 0 &&
-         pl->beam_stride % 16 == 0 && (reinterpret_cast<uintptr_t>(d_data) & 15) == 0 &&
+         u8_ring_depth(p.n_beam) >= 2 && p.n_samp_sub % kT == 0 && p.n_samp_sub <= 1024 &&
+         p.n_chan % kBoxCh == 0 && pl->beam_stride % 16 == 0 &&
+         (reinterpret_cast<uintptr_t>(d_data) & 15) == 0 &&
          (int64_t)p.n_sub * p.n_samp_sub <= 2147483647ll /* TMA time coordinate */ &&
          encode_fn() != nullptr;
 }
 
-cudaError_t launch_gram_tc(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
-                           int64_t* d_sums, float* d_corr, int64_t* d_sums8, int n_pol) {
+cudaError_t launch_gram_tc_pol2(const mraid_plan_s* pl, const uint8_t* d_data, int64_t* d_sums,
+                                float* d_corr) {
   const mraid_params& p = pl->p;
-  if (!gram_tc_supported(pl, d_data, n_pol)) return cudaErrorNotSupported;
-  const int variant = tc_variant_for(pl, n_pol);
+  if (!gram_tc_pol2_supported(pl, d_data)) return cudaErrorNotSupported;
   CUtensorMap map;
-  const cuuint64_t n_time = (cuuint64_t)(sub0 + n_sub) * p.n_samp_sub;
-  // one box holds every block of the stage: n_pol * N blocks, beam_stride apart
-  cuuint64_t dims[3] = {(cuuint64_t)p.n_chan, n_time, (cuuint64_t)n_pol * p.n_beam};
+  const cuuint64_t n_time = (cuuint64_t)p.n_sub * p.n_samp_sub;
+  // one box holds every block of the stage: 2 N blocks, beam_stride apart
+  cuuint64_t dims[3] = {(cuuint64_t)p.n_chan, n_time, (cuuint64_t)2 * p.n_beam};
   cuuint64_t strides[2] = {(cuuint64_t)p.n_chan, (cuuint64_t)pl->beam_stride};
-  const int t = tc_variant_samples(variant);
-  cuuint32_t box[3] = {(cuuint32_t)kBoxCh, (cuuint32_t)t, (cuuint32_t)(n_pol * p.n_beam)};
+  cuuint32_t box[3] = {(cuuint32_t)kBoxCh, (cuuint32_t)kT, (cuuint32_t)(2 * p.n_beam)};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = encode_fn()(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(d_data),
                            dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1555,77 +869,35 @@ cudaError_t launch_gram_tc(const mraid_plan_s* pl, const uint8_t* d_data, int su
   a.n_beam = p.n_beam;
   a.n_chan = p.n_chan;
   a.n_samp_sub = p.n_samp_sub;
-  a.sub0 = sub0;
-  a.n_sub = n_sub;
-  a.n_pol = n_pol;
-  a.center = n_pol == 2 ? 255 : 128;
-  // FP32 sums in TMEM stay exact while they are below 2^24: 1024 samples of
-  // products up to 128^2 for one polarisation, 256 samples of products up to
-  // 255^2 for the sum of two; a sub-integration of two polarisations is
-  // accumulated in pieces (the largest number of stages dividing it within
-  // 256 samples) that the epilogue adds as integers
+  a.sub0 = 0;
+  a.n_sub = p.n_sub;
+  // FP32 sums in TMEM stay exact below 2^24: 256 samples of products up to
+  // 255^2. A sub-integration is accumulated in pieces (the largest number of
+  // stages dividing it within 256 samples) that the epilogue adds as integers
   {
-    const int stages = p.n_samp_sub / t;
+    const int stages = p.n_samp_sub / kT;
     int d = stages;
-    if (n_pol == 2)
-      while (d > 1 && (stages % d != 0 || d * t > 256)) --d;
+    while (d > 1 && (stages % d != 0 || d * kT > 256)) --d;
     a.piece_stages = d;
   }
-  const int R = p.n_beam + 1;              // beams + the row of ones
+  const int R = p.n_beam + 1;  // beams + the row of ones
   a.R = R;
   a.R2 = R > 16 ? R - 16 : 0;
-  a.rb = (R + 1) / 2 * 2;                  // B of the first MMAs: R slots, even count
-  a.sums = d_sums8 ? nullptr : d_sums;
-  a.sums8 = d_sums8;
+  a.rb = (R + 1) / 2 * 2;  // B of the first MMAs: R slots, even count
+  a.sums = d_sums;
   a.corr = d_corr;
   a.degenerate = pl->d_degenerate;
   a.error = pl->d_error;
   a.wait_ns = pl->wait_ns;
   a.withhold = pl->inject_withhold;
-  const int64_t items = (int64_t)n_sub * (p.n_chan / kBoxCh);
+  a.n_u8 = u8_ring_depth(p.n_beam);
+  const size_t smem = smem_bytes(p.n_beam, a.n_u8);
+  const int64_t items = (int64_t)p.n_sub * (p.n_chan / kBoxCh);
   const int grid = (int)(items < pl->sm_count ? items : pl->sm_count);
-  cudaError_t e = cudaSuccess;
-#define MRAID_TC_LAUNCH_P(T, NF, U, P)                                                             \
-  do {                                                                                           \
-    using C_ = TcCfg<T, NF, U>;                                                                     \
-    const int n_u8 = u8_ring_depth<C_>(p.n_beam, P);                                             \
-    a.n_u8 = n_u8;                                                                               \
-    const size_t smem = smem_bytes<C_>(p.n_beam, n_u8, P);                                       \
-    e = cudaFuncSetAttribute(gram_tc_kernel<T, NF, U, P>,                                        \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);           \
-    if (e == cudaSuccess && grid > 0)                                                            \
-      gram_tc_kernel<T, NF, U, P><<<grid, kThreads, smem, pl->stream>>>(map, a);                  \
-  } while (0)
-#define MRAID_TC_LAUNCH(T, NF, U) MRAID_TC_LAUNCH_P(T, NF, U, 1)
-#define MRAID_TCA_LAUNCH(T)                                                                       \
-  do {                                                                                           \
-    const int na_ = tca_sub_stages(a.rb, a.R2);                                                  \
-    const int n_u8 = tca_u8_depth<T>(p.n_beam, na_);                                             \
-    a.n_u8 = n_u8;                                                                               \
-    const size_t smem = tca_smem_bytes<T>(p.n_beam, na_, n_u8);                                  \
-    e = cudaFuncSetAttribute(gram_tc_a_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                             (int)smem);                                                        \
-    if (e == cudaSuccess && grid > 0)                                                            \
-      gram_tc_a_kernel<T><<<grid, kThreads, smem, pl->stream>>>(map, a);                          \
-  } while (0)
-  if (n_pol == 2) {
-    MRAID_TC_LAUNCH_P(64, 2, 1, 2);  // variant 0: two f16 stages leave room for the doubled u8 ring
-  } else switch (variant) {
-    case 8: MRAID_TCA_LAUNCH(64); break;
-    case 9: MRAID_TCA_LAUNCH(32); break;
-    case 1: MRAID_TC_LAUNCH(32, 4, 1); break;
-    case 2: MRAID_TC_LAUNCH(32, 2, 1); break;
-    case 3: MRAID_TC_LAUNCH(64, 3, 1); break;
-    case 4: MRAID_TC_LAUNCH(64, 2, 2); break;
-    case 5: MRAID_TC_LAUNCH(64, 3, 2); break;
-    case 6: MRAID_TC_LAUNCH(64, 4, 1); break;
-    case 7: MRAID_TC_LAUNCH(64, 4, 2); break;
-    default: MRAID_TC_LAUNCH(64, 2, 1); break;
-  }
-#undef MRAID_TC_LAUNCH
-#undef MRAID_TC_LAUNCH_P
-#undef MRAID_TCA_LAUNCH
+  cudaError_t e = cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
   if (e != cudaSuccess) return e;
+  if (grid > 0) gram_tc_kernel<<<grid, kThreads, smem, pl->stream>>>(map, a);
   return cudaGetLastError();
 }
 
@@ -1662,11 +934,8 @@ cudaError_t launch_gram_tc_f32(const mraid_plan_s* pl, const float* d_data, int 
   a.R = R;
   a.R2 = R > 16 ? R - 16 : 0;
   a.rb = (R + 1) / 2 * 2;
-  a.n_pol = 1;
-  a.center = 0;
   a.piece_stages = 1;
   a.sums = nullptr;
-  a.sums8 = nullptr;
   a.corr = d_corr;
   a.degenerate = pl->d_degenerate;
   a.error = pl->d_error;

@@ -89,7 +89,8 @@ struct mraid_plan_s {
   cudaEvent_t ev_consumed[2] = {nullptr, nullptr};
   mraid::Profiler prof;
   bool force_dp4a = false;  // use the CUDA-core Gram even where tcgen05 fits
-  int tc_variant = 0;       // tensor-core Gram variant (tc_default_variant, or autotuned)
+  int tc_variant = 0;       // 8-bit Gram up to 23 beams: even = work items by the shape,
+                            // odd = always of 64 channels
   unsigned long long wait_ns = 2000000000ull;  // bound of every device wait
   long long inject_withhold = -1;  // MRAID_FAULT_WITHHOLD_STAGE: stage to skip, or -1
   bool inject_alloc = false;       // MRAID_FAULT_ALLOC armed
@@ -143,11 +144,6 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
                        int64_t* d_sums, float* d_corr);
 // copy the device masking report to the caller's struct at the next sync
 mraid_status enqueue_info_copy(mraid_plan_s* pl, mraid_flag_info* info);
-// one pass over 8-bit samples: the Gram sums of every sub-integration into
-// ws.sums (interleaved by 8 channels when the tensor cores form them), and
-// the correlation into d_corr when it is not null
-mraid_status gram_sums_pass(mraid_plan_s* pl, const void* d_data, float* d_corr,
-                            bool* interleaved);
 // Allocate every work buffer mraid_run can need (so later calls allocate
 // nothing, e.g. inside a stream capture).
 mraid_status plan_prepare(mraid_plan_s* pl);
@@ -176,24 +172,13 @@ cudaError_t launch_gram_u8(const mraid_plan_s* pl, const uint8_t* d_data,
 // float32 samples: correlation on CUDA cores (d_corr relative to sub0)
 cudaError_t launch_gram_f32(const mraid_plan_s* pl, const float* d_data, int sub0, int n_sub,
                             float* d_corr);
-// tensor-core Gram fused with the correlation (gram_tc.cu); either output
-// may be null. cudaErrorNotSupported when the shape or layout does not fit.
-// n_pol 2: blocks b and N + b are two polarisations of beam b, summed in
-// the converter; the sums and the correlation are of the total power (exact:
-// TMEM accumulates pieces of at most 256 samples, the epilogue adds them)
-bool gram_tc_supported(const mraid_plan_s* pl, const void* d_data, int n_pol = 1);
-int tc_variant_samples(int v);
-int tc_default_variant(int n_beam);
-constexpr int kTcVariants = 10;
-// the tensor-core variant a plan's launch runs (variants 8 and 9 fall back
-// to the default where their A-in-TMEM kernel does not fit the shape)
-int tc_variant_effective(const mraid_plan_s* pl);
+// gram_tc.cu: two polarisations (blocks b and N + b of beam b) added as they
+// are read; sums and correlation (either may be null) are of the total power
+bool gram_tc_pol2_supported(const mraid_plan_s* pl, const void* d_data);
+cudaError_t launch_gram_tc_pol2(const mraid_plan_s* pl, const uint8_t* d_data, int64_t* d_sums,
+                                float* d_corr);
+constexpr int kTcVariants = 10;  // 8-bit tensor-core Gram ids (see tc_variant)
 constexpr int kEigVariants = 6;  // register eigensolvers (see eig_variant)
-// d_sums8 (instead of d_sums): the sums in the interleaved layout
-// [cell / 8][P][cell % 8], which the kernel writes in 64-byte runs
-cudaError_t launch_gram_tc(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
-                           int64_t* d_sums, float* d_corr, int64_t* d_sums8 = nullptr,
-                           int n_pol = 1);
 // float32 samples on the tensor cores (split-bf16 products, gram_tc.cu):
 // correlation only, d_corr relative to sub0
 // Tensor-core Gram for 24..127 beams, one channel per MMA (gram_tcl.cu):
@@ -202,12 +187,20 @@ cudaError_t launch_gram_tc(const mraid_plan_s* pl, const uint8_t* d_data, int su
 bool gram_tcl_supported(const mraid_plan_s* pl, const void* d_data);
 cudaError_t launch_gram_tcl(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
                             int64_t* d_sums);
+// gram_mma.cu: 8-bit Gram for up to 23 beams, any layout, fused with the
+// correlation (sub-integrations of up to gram_mma_piece samples; longer ones
+// give the sums only). gram_mma_bulk: true where the samples come by bulk
+// tensor copies.
+constexpr int kMmPieceMax = 1024;
+bool gram_mma_supported(const mraid_plan_s* pl);
+bool gram_mma_bulk(const mraid_plan_s* pl, const void* d_data);
+cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
+                            int64_t* d_sums, float* d_corr);
 bool gram_tc_f32_supported(const mraid_plan_s* pl, const void* d_data);
 cudaError_t launch_gram_tc_f32(const mraid_plan_s* pl, const float* d_data, int sub0, int n_sub,
                                float* d_corr);
-// interleaved: d_sums in the [cell / 8][P][cell % 8] layout
 cudaError_t launch_corr_from_sums(const mraid_plan_s* pl, const int64_t* d_sums,
-                                  int64_t n_cells, float* d_corr, bool interleaved = false);
+                                  int64_t n_cells, float* d_corr);
 // eig.cu
 cudaError_t launch_eig(const mraid_plan_s* pl, const float* d_corr, int64_t n_cells,
                        float* d_evals, float* d_q1, float* d_stat);
@@ -248,11 +241,9 @@ cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, i
                          double ratio, int itermax, double* d_z, float* d_zf, int32_t* d_iters,
                          double* d_work);
 // time-aggregated spectra [interval][beam][chan] from the Gram sums
-cudaError_t launch_bandpass_input(const mraid_plan_s* pl, const int64_t* d_sums, bool interleaved,
-                                  int interval, double* d_y);
+cudaError_t launch_bandpass_input(const mraid_plan_s* pl, const int64_t* d_sums, int interval, double* d_y);
 // per cell C_ab = cov_ab / n^2 + (mu_a - z_a)(mu_b - z_b), packed, all cells
-cudaError_t launch_ccm_bandpass(const mraid_plan_s* pl, const int64_t* d_sums, bool interleaved,
-                                int interval, const double* d_z, float* d_ccm);
+cudaError_t launch_ccm_bandpass(const mraid_plan_s* pl, const int64_t* d_sums, int interval, const double* d_z, float* d_ccm);
 // pol2.cu: total-power sums [cell][P] from the stacked 2N-block sums
 cudaError_t launch_pol2_fold(const mraid_plan_s* pl, const int64_t* d_stacked, int64_t n_cells,
                              int64_t* d_sums);

@@ -153,12 +153,9 @@ mraid_status mraid_multires(mraid_plan_t pl, const void* d_data, int32_t n_level
   if (e == cudaSuccess) e = reset_counters();
   if (e != cudaSuccess) return cuda_fail(e, "memset");
   // the one pass over the samples: Gram sums of every sub-integration, and
-  // the correlation too when the plan's own length is a level; the
-  // aggregation adds whole sub-integrations, so it does not depend on the
-  // sums' layout, and the correlation kernel reads either
+  // the correlation too when the plan's own length is a level
   const bool has1 = factors[order[0]] == 1;
-  bool inter = false;
-  st = gram_sums_pass(pl, d_data, has1 ? pl->ws.corr : nullptr, &inter);
+  st = ccm_range(pl, d_data, 0, n_sub, pl->ws.sums, has1 ? pl->ws.corr : nullptr);
   if (st != MRAID_OK) return st;
   for (int li = 0; li < n_levels; ++li) {
     const int i = order[li], f = factors[i];
@@ -180,7 +177,7 @@ mraid_status mraid_multires(mraid_plan_t pl, const void* d_data, int32_t n_level
       if (e == cudaSuccess)
         e = MRAID_PROF(pl, K_AGG, launch_gram_aggregate(pl, src, dst, n_f, f / g));
       if (e == cudaSuccess)
-        e = MRAID_PROF(pl, K_CORR, launch_corr_from_sums(pl, dst, cells, pl->ws.corr, inter));
+        e = MRAID_PROF(pl, K_CORR, launch_corr_from_sums(pl, dst, cells, pl->ws.corr));
       if (e != cudaSuccess) return cuda_fail(e, "multires sums");
     }
     e = MRAID_PROF(pl, K_EIG, launch_eig(pl, pl->ws.corr, cells, nullptr, nullptr, d_stats[i]));

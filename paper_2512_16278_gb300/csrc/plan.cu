@@ -224,11 +224,14 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
     }
     return MRAID_OK;
   }
-  if (!pl->force_dp4a && gram_tc_supported(pl, d_data)) {
-    cudaError_t e = MRAID_PROF(pl, K_GRAM_TC,
-                               launch_gram_tc(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
-                                              d_sums, d_corr));
-    return e == cudaSuccess ? MRAID_OK : cuda_fail(e, "gram_tc launch");
+  const bool mma = !pl->force_dp4a && gram_mma_supported(pl);
+  // profiled by the way the samples come: "gram_tc" for bulk tensor copies
+  const int mma_id = mma && gram_mma_bulk(pl, d_data) ? K_GRAM_TC : K_GRAM;
+  if (mma && pl->p.n_samp_sub <= kMmPieceMax) {
+    cudaError_t e = MRAID_PROF(pl, mma_id,
+                               launch_gram_mma(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
+                                               d_sums, d_corr));
+    return e == cudaSuccess ? MRAID_OK : cuda_fail(e, "gram_mma launch");
   }
   int64_t* sums = d_sums;
   if (!sums) {
@@ -236,7 +239,12 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
     if (st != MRAID_OK) return st;
     sums = pl->ws.sums;
   }
-  if (!pl->force_dp4a && gram_tcl_supported(pl, d_data)) {
+  if (mma) {
+    cudaError_t e = MRAID_PROF(pl, mma_id,
+                               launch_gram_mma(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
+                                               sums, nullptr));
+    if (e != cudaSuccess) return cuda_fail(e, "gram_mma launch");
+  } else if (!pl->force_dp4a && gram_tcl_supported(pl, d_data)) {
     cudaError_t e = MRAID_PROF(pl, K_GRAM_TCL,
                                launch_gram_tcl(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
                                                sums));
@@ -263,23 +271,6 @@ mraid_status enqueue_info_copy(mraid_plan_s* pl, mraid_flag_info* info) {
   if (e != cudaSuccess) return cuda_fail(e, "info copy");
   pl->pending_info = info;
   return MRAID_OK;
-}
-
-// One pass over 8-bit samples for the paths that need the Gram sums: the
-// int64 sums of every sub-integration into ws.sums (and the correlation
-// into d_corr when it is not null). The tensor-core kernel writes the sums
-// interleaved by 8 channels ([cell / 8][P][cell % 8], 64-byte store runs;
-// *interleaved = true); otherwise they are [cell][P].
-mraid_status gram_sums_pass(mraid_plan_s* pl, const void* d_data, float* d_corr,
-                            bool* interleaved) {
-  *interleaved = !pl->force_dp4a && gram_tc_supported(pl, d_data);
-  if (*interleaved) {
-    cudaError_t e = MRAID_PROF(pl, K_GRAM_TC,
-                               launch_gram_tc(pl, static_cast<const uint8_t*>(d_data), 0,
-                                              pl->p.n_sub, nullptr, d_corr, pl->ws.sums));
-    return e == cudaSuccess ? MRAID_OK : cuda_fail(e, "gram_tc launch");
-  }
-  return ccm_range(pl, d_data, 0, pl->p.n_sub, pl->ws.sums, d_corr);
 }
 
 mraid_status plan_prepare(mraid_plan_s* pl) {
@@ -423,7 +414,6 @@ mraid_status mraid_plan(const mraid_params* p, void* stream, mraid_plan_t* out) 
   }
   pl->p = *p;
   pl->p.keep = nullptr;
-  pl->tc_variant = tc_default_variant(p->n_beam);
   pl->stream = static_cast<cudaStream_t>(stream);
   pl->n_cells = (int64_t)p->n_sub * p->n_chan;
   pl->beam_stride = p->beam_stride ? p->beam_stride : (int64_t)p->n_sub * p->n_samp_sub * p->n_chan;
@@ -796,9 +786,8 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
     // float32 samples, and 24..127 beams, have one tensor-core kernel each,
     // timed as variant 0
     if (v >= 0 && (pl->p.bit_depth == 32 ? (v > 0 || !gram_tc_f32_supported(pl, d_data))
-                   : gram_tcl_supported(pl, d_data) ? v > 0
-                                                    : (!gram_tc_supported(pl, d_data) ||
-                                                       tc_variant_effective(pl) != v)))
+                                           : (!gram_mma_supported(pl) &&
+                                              (v > 0 || !gram_tcl_supported(pl, d_data)))))
       continue;
     float ms = 0.f;
     st = time_runs(pl, reps, e0, e1,

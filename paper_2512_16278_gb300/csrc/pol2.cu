@@ -72,7 +72,7 @@ namespace {
 // sub-integration in its epilogue, so it writes the total power's sums
 // and correlation directly.
 bool pol2_on_tensor_cores(const mraid_plan_s* pl, const void* d_data) {
-  return !pl->force_dp4a && pl->p.bit_depth == 8 && gram_tc_supported(pl, d_data, 2);
+  return !pl->force_dp4a && pl->p.bit_depth == 8 && gram_tc_pol2_supported(pl, d_data);
 }
 
 // Otherwise: the exact 8-bit Gram of the 2N stacked blocks (a plan view
@@ -106,12 +106,11 @@ mraid_status pol2_stacked_sums(mraid_plan_s* pl, const void* d_data, int64_t* d_
   v.d_degenerate = pl->d_degenerate;
   v.d_error = pl->d_error;
   v.force_dp4a = pl->force_dp4a;
-  v.tc_variant = tc_default_variant(2 * N);
   cudaError_t e = cudaSuccess;
-  if (!v.force_dp4a && gram_tc_supported(&v, d_data)) {
-    e = MRAID_PROF(pl, K_GRAM_TC,
-                   launch_gram_tc(&v, static_cast<const uint8_t*>(d_data), 0, v.p.n_sub,
-                                  pl->pol_sums, nullptr));
+  if (!v.force_dp4a && gram_mma_supported(&v)) {
+    e = MRAID_PROF(pl, gram_mma_bulk(&v, d_data) ? K_GRAM_TC : K_GRAM,
+                   launch_gram_mma(&v, static_cast<const uint8_t*>(d_data), 0, v.p.n_sub,
+                                   pl->pol_sums, nullptr));
   } else {
     for (int s = 0; s < v.p.n_sub && e == cudaSuccess; s += kMaxSubPerLaunch) {
       const int ns = (v.p.n_sub - s) < kMaxSubPerLaunch ? (v.p.n_sub - s) : kMaxSubPerLaunch;
@@ -140,8 +139,8 @@ mraid_status pol2_ccm(mraid_plan_s* pl, const void* d_data, int64_t* d_sums, flo
   if (e != cudaSuccess) return cuda_fail(e, "memset");
   if (pol2_on_tensor_cores(pl, d_data)) {
     e = MRAID_PROF(pl, K_GRAM_TC,
-                   launch_gram_tc(pl, static_cast<const uint8_t*>(d_data), 0, pl->p.n_sub, d_sums,
-                                  d_corr, nullptr, 2));
+                   launch_gram_tc_pol2(pl, static_cast<const uint8_t*>(d_data), d_sums,
+                                       d_corr));
     return e == cudaSuccess ? MRAID_OK : cuda_fail(e, "gram_tc launch");
   }
   int64_t* sums = d_sums;
