@@ -70,6 +70,7 @@ struct mraid_plan_s {
   uint8_t* d_keep = nullptr;          // [n_chan]
   double* d_partials = nullptr;       // flag partial sums [2][blocks][3]
   int flag_blocks = 0;
+  int flag_ctas = 0;                  // widest cluster of the cluster masking kernel (0: none)
   mraid_flag_info* d_info = nullptr;  // device flag info
   unsigned long long* d_degenerate = nullptr;
   unsigned* d_error = nullptr;        // device error word (bounded waits)
@@ -252,5 +253,6 @@ cudaError_t launch_pol2_fold(const mraid_plan_s* pl, const int64_t* d_stacked, i
 cudaError_t launch_gram_aggregate(const mraid_plan_s* pl, const int64_t* d_src, int64_t* d_dst,
                                   int n_out_sub, int m);
 int flag_grid_blocks(int device, int sm_count);
+int flag_cluster_ctas(int device);
 
 }  // namespace mraid

@@ -424,6 +424,7 @@ mraid_status mraid_plan(const mraid_params* p, void* stream, mraid_plan_t* out) 
   if (e == cudaSuccess) {
     pl->flag_blocks = flag_grid_blocks(pl->device, pl->sm_count);
     if (pl->flag_blocks < 1) e = cudaErrorLaunchOutOfResources;
+    pl->flag_ctas = flag_cluster_ctas(pl->device);
   }
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_partials, sizeof(double) * 6 * (size_t)pl->flag_blocks);
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_info, sizeof(mraid_flag_info));
