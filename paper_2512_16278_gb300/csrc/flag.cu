@@ -288,6 +288,12 @@ __device__ __forceinline__ void cl_sync() {
       "barrier.cluster.wait.acquire.aligned;" ::
           : "memory");
 }
+// A pivot near c: eight significant bits, so that rounding v - pivot depends
+// on v's low bits alone and does not lean one way over cells of like values;
+// no shift for infinities and NaN.
+__device__ __forceinline__ float pivot_near(float c) {
+  return fabsf(c) < 1e30f ? __uint_as_float(__float_as_uint(c) & 0xffff0000u) : 0.f;
+}
 // s + e = a + b exactly (Knuth's two-sum)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;
@@ -380,7 +386,7 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
     const ClPart p = block3(ClPart{use ? 1.f : 0.f, v, 0.f, 0.f});
     if (tid == 0) {
       const float c = p.s1 / fmaxf(p.n, 1.f);
-      fit_pivot = fabsf(c) < 1e30f ? c : 0.f;  // infinities and NaN: no shift
+      fit_pivot = pivot_near(c);
     }
     __syncthreads();
   }
@@ -444,8 +450,7 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
       }
       fit_thresh = thresh;
       fit_stop = stop;
-      const float c = (float)mu;
-      fit_pivot = fabsf(c) < 1e30f ? c : 0.f;
+      fit_pivot = pivot_near((float)mu);
     }
     __syncthreads();
     thresh = fit_thresh;
