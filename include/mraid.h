@@ -83,7 +83,8 @@ typedef struct {
   int64_t n_degenerate;  /* (beam, cell) pairs with zero variance (mraid_run) */
   int64_t jacobi_sweeps; /* eigensolver iterations summed over cells (mraid_run; 0 if not
                             counted): Jacobi sweeps, or implicit QR steps for the
-                            tridiagonal variant */
+                            tridiagonal variants (the split ones run QR, and count,
+                            only when eigenvalues or q1 are asked for) */
   int64_t jacobi_warp_sweeps; /* the same, as executed: each 32-cell warp counts its slowest
                                  cell (mraid_run) */
   int32_t timed_out;     /* 1 if a bounded device wait expired */

@@ -844,14 +844,23 @@ eig_tri_kernel(const float* __restrict__ corr, int64_t n_cells, float* __restric
 // monotonically to lambda_1, so sigma = lambda_1 + delta for the inverse
 // iteration stays above it. It then computes q1 while the reflectors are in
 // its shared memory. A second kernel with a few dozen registers runs QR on
-// T for all eigenvalues at several times the occupancy.
-constexpr int kNewtonMax = 40;
+// T for all eigenvalues at several times the occupancy; it only runs when the
+// caller wants them: the statistic needs lambda_1 and sum lambda_i^2 =
+// ||T||_F^2, which the first kernel has. Measured on GB300: 1 024 cells of 19
+// beams without eigenvalues 60 -> 27 us, the seven timescales (301 056 cells)
+// 2.26 -> 1.96 ms per call; the statistic's error against 64 bits falls from
+// 5e-6 to 4e-7 there (the QR's deflation bound no longer enters it). With
+// eigenvalues and no q1 the Newton loop costs 5 % (155 648 cells of 13 beams
+// 20 us), so that the statistic is the same bits whatever else is asked for.
+// Newton's steps shrink by 1 - 1/m at an m-fold lambda_1: the bound lets an
+// 18-fold one converge to 1e-7 (282 steps); a simple one takes about ten.
+constexpr int kNewtonMax = 400;
 constexpr int kEigQrThreads = 128;
 
 template <int N>
 __global__ void __launch_bounds__(kEigThreads)
 eig_tri_a_kernel(const float* __restrict__ corr, int64_t n_cells, float* __restrict__ de,
-                 float* __restrict__ q1) {
+                 float* __restrict__ q1, float* __restrict__ stat) {
   constexpr int NP = Slots<N>::NP;
   constexpr int STR = Slots<N>::STR;
   extern __shared__ float sm[];
@@ -934,12 +943,12 @@ eig_tri_a_kernel(const float* __restrict__ corr, int64_t n_cells, float* __restr
   if (!active) return;
   const int64_t cell = cell0 + threadIdx.x;
   // T for the QR kernel, d then e, one row of n_cells floats per entry
-  static_for<N>([&](auto ii) {
-    constexpr int i = decltype(ii)::value;
-    de[(int64_t)i * n_cells + cell] = td[i];
-    de[(int64_t)(N + i) * n_cells + cell] = te[i];
-  });
-  if (!q1) return;
+  if (de)
+    static_for<N>([&](auto ii) {
+      constexpr int i = decltype(ii)::value;
+      de[(int64_t)i * n_cells + cell] = td[i];
+      de[(int64_t)(N + i) * n_cells + cell] = te[i];
+    });
   // lambda_1 of T: Newton on det(T - x I) from Gershgorin's upper bound
   float lam = -3.0e38f;
   static_for<N>([&](auto ii) {
@@ -970,6 +979,17 @@ eig_tri_a_kernel(const float* __restrict__ corr, int64_t n_cells, float* __restr
     lam -= step;
     if (!(step > 1e-7f * fabsf(lam))) break;
   }
+
+  {
+    float ss = 0.f;
+    static_for<N>([&](auto ii) {
+      constexpr int i = decltype(ii)::value;
+      ss = fmaf(td[i], td[i], ss);
+      if constexpr (i < N - 1) ss = fmaf(2.f * te[i], te[i], ss);
+    });
+    stat[cell] = ss > 0.f ? lam * lam / ss : 0.f;
+  }
+  if (!q1) return;
 
   // q1: inverse iteration with sigma I - T = L D L^T (sigma just above
   // lambda_1, so every pivot is positive), then x = Q y.
@@ -1046,7 +1066,7 @@ eig_tri_a_kernel(const float* __restrict__ corr, int64_t n_cells, float* __restr
 template <int N, bool kCompact, bool kRootFree = false>
 __global__ void __launch_bounds__(kEigQrThreads)
 eig_qr_kernel(const float* __restrict__ de, int64_t n_cells, float* __restrict__ evals,
-              float* __restrict__ stat, unsigned long long* __restrict__ step_count) {
+              unsigned long long* __restrict__ step_count) {
   const int64_t cell = (int64_t)blockIdx.x * kEigQrThreads + threadIdx.x;
   const bool active = cell < n_cells;
   float d[N], e[N];
@@ -1164,10 +1184,7 @@ eig_qr_kernel(const float* __restrict__ de, int64_t n_cells, float* __restrict__
     });
   });
   if (!active) return;
-  float ss = 0.f;
-  static_for<N>([&](auto kk) { ss = fmaf(d[decltype(kk)::value], d[decltype(kk)::value], ss); });
-  stat[cell] = ss > 0.f ? d[0] * d[0] / ss : 0.f;
-  if (evals) static_for<N>([&](auto kk) { evals[cell * N + decltype(kk)::value] = d[decltype(kk)::value]; });
+  static_for<N>([&](auto kk) { evals[cell * N + decltype(kk)::value] = d[decltype(kk)::value]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -1445,16 +1462,16 @@ cudaError_t launch_reg(const float* d_corr, int64_t n_cells, float* d_evals, flo
                              (int)smem);
     if (e != cudaSuccess) return e;
     if (blocks > 0)
-      eig_tri_a_kernel<N><<<(unsigned)blocks, kEigThreads, smem, stream>>>(d_corr, n_cells, d_de,
-                                                                             d_q1);
-    const int64_t qb = (n_cells + kEigQrThreads - 1) / kEigQrThreads;
+      eig_tri_a_kernel<N><<<(unsigned)blocks, kEigThreads, smem, stream>>>(
+          d_corr, n_cells, d_evals ? d_de : nullptr, d_q1, d_stat);
+    const int64_t qb = d_evals ? (n_cells + kEigQrThreads - 1) / kEigQrThreads : 0;
     if (qb > 0) {
       if (variant == 5)
         eig_qr_kernel<N, true, true><<<(unsigned)qb, kEigQrThreads, 0, stream>>>(
-            d_de, n_cells, d_evals, d_stat, sweep_count);
+            d_de, n_cells, d_evals, sweep_count);
       else
         eig_qr_kernel<N, true><<<(unsigned)qb, kEigQrThreads, 0, stream>>>(d_de, n_cells, d_evals,
-                                                                             d_stat, sweep_count);
+                                                                             sweep_count);
     }
     return cudaGetLastError();
   }
