@@ -19,11 +19,14 @@
 // cov_ab = n S_ab - S_a S_b the exact int64 covariance numerator and
 // d_a = S_a / n - z_a the cell mean's offset from the bandpass: no
 // cancellation between large terms, so FP32 suffices for C.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace mraid {
 namespace {
@@ -32,18 +35,38 @@ constexpr int kArThreads = 512;
 constexpr int kArWarps = kArThreads / 32;
 constexpr int kCrArrays = 13;  // per block row: A (3), C (4), saved left coupling (4), F (2)
 
-// Sum over the block in a fixed order; every thread gets the total.
-__device__ double block_sum(double v, double* red) {
+// Sums of two values over the block in a fixed order; every thread gets the
+// totals. One warp adds the warps' sums: FP64 issue is scarce (two lanes per
+// cycle and SM on GB300), and every warp adding all 16 cost 2 us a sum.
+__device__ void block_sum2(double& a, double& b, double (*red)[2]) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   __syncthreads();
-  if (lane == 0) red[warp] = v;
+  if (lane == 0) {
+    red[warp][0] = a;
+    red[warp][1] = b;
+  }
   __syncthreads();
-  double t = 0.0;
-#pragma unroll 8
-  for (int i = 0; i < kArWarps; ++i) t += red[i];
-  return t;
+  if (warp == 0) {
+    a = lane < kArWarps ? red[lane][0] : 0.0;
+    b = lane < kArWarps ? red[lane][1] : 0.0;
+#pragma unroll
+    for (int o = kArWarps / 2; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) {
+      red[kArWarps][0] = a;
+      red[kArWarps][1] = b;
+    }
+  }
+  __syncthreads();
+  a = red[kArWarps][0];
+  b = red[kArWarps][1];
 }
 
 // Entries of D^T D for D the (n-2) x n second-difference matrix (rows
@@ -86,96 +109,176 @@ struct CrArrays {  // m block rows each
 // rows are recovered level by level. It is Gaussian elimination of the
 // symmetric positive definite matrix in an odd-even order, so it needs no
 // pivoting, and every level is parallel over its rows.
-__device__ void cr_solve(const CrArrays& r, int m, const double* w, const double* y, int n,
-                         double lam) {
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const int r0 = 2 * i, r1 = 2 * i + 1;
+//
+// A cluster of K CTAs shares one spectrum: CTA r holds block rows [r mk,
+// (r + 1) mk), mk = m / K. A level reads one row of the CTA before (the last
+// leaving one); when one row per CTA is left, CTA 0 solves those K rows.
+
+// Row j leaves: its A becomes the inverse, its left coupling is kept.
+__device__ __forceinline__ void cr_leave(const CrArrays& r, int j, const M2& Cprev) {
+  const double a = r.aa[j], b = r.ab[j], d = r.ad[j];
+  const double inv = 1.0 / fma(a, d, -b * b);
+  r.aa[j] = d * inv;
+  r.ab[j] = -b * inv;
+  r.ad[j] = a * inv;
+  const M2 L = tr(Cprev);
+  r.l00[j] = L.a;
+  r.l01[j] = L.b;
+  r.l10[j] = L.c;
+  r.l11[j] = L.d;
+}
+
+// Row i takes in the row before it (rp, jp; jp < 0: none) and the row jn after it
+// (jn < 0: none).
+__device__ __forceinline__ void cr_stay(const CrArrays& r, int i, const CrArrays& rp, int jp,
+                                        int jn) {
+  M2 Ai = r.A(i);
+  double g0 = r.f0[i], g1 = r.f1[i];
+  if (jp >= 0) {
+    const M2 Cj = rp.C(jp);
+    M2 al = mm(tr(Cj), rp.A(jp));
+    al = {-al.a, -al.b, -al.c, -al.d};
+    const M2 t = mm(al, Cj);
+    Ai = {Ai.a + t.a, Ai.b + t.b, Ai.c + t.c, Ai.d + t.d};
+    g0 = fma(al.a, rp.f0[jp], fma(al.b, rp.f1[jp], g0));
+    g1 = fma(al.c, rp.f0[jp], fma(al.d, rp.f1[jp], g1));
+  }
+  M2 Cn = {0.0, 0.0, 0.0, 0.0};
+  if (jn >= 0) {
+    const M2 Ci = r.C(i);
+    M2 ga = mm(Ci, r.A(jn));
+    ga = {-ga.a, -ga.b, -ga.c, -ga.d};
+    const M2 t = mm(ga, tr(Ci));
+    Ai = {Ai.a + t.a, Ai.b + t.b, Ai.c + t.c, Ai.d + t.d};
+    g0 = fma(ga.a, r.f0[jn], fma(ga.b, r.f1[jn], g0));
+    g1 = fma(ga.c, r.f0[jn], fma(ga.d, r.f1[jn], g1));
+    Cn = mm(ga, r.C(jn));
+  }
+  r.aa[i] = Ai.a;
+  r.ab[i] = 0.5 * (Ai.b + Ai.c);
+  r.ad[i] = Ai.d;
+  r.c00[i] = Cn.a;
+  r.c01[i] = Cn.b;
+  r.c10[i] = Cn.c;
+  r.c11[i] = Cn.d;
+  r.f0[i] = g0;
+  r.f1[i] = g1;
+}
+
+// The eliminated row j from the solutions before it (row j - s) and after
+// it: row j + s, or (y0, y1) of the next CTA's first row.
+__device__ __forceinline__ void cr_back(const CrArrays& r, int j, int s, int m, double y0, double y1) {
+  const double x0 = r.f0[j - s], x1 = r.f1[j - s];
+  double g0 = r.f0[j] - fma(r.l00[j], x0, r.l01[j] * x1);
+  double g1 = r.f1[j] - fma(r.l10[j], x0, r.l11[j] * x1);
+  if (j + s < m) {
+    y0 = r.f0[j + s];
+    y1 = r.f1[j + s];
+  }
+  g0 -= fma(r.c00[j], y0, r.c01[j] * y1);
+  g1 -= fma(r.c10[j], y0, r.c11[j] * y1);
+  r.f0[j] = fma(r.aa[j], g0, r.ab[j] * g1);
+  r.f1[j] = fma(r.ab[j], g0, r.ad[j] * g1);
+}
+
+__device__ __forceinline__ void cr_last(const CrArrays& r) {  // the one row left
+  const double a = r.aa[0], b = r.ab[0], d = r.ad[0];
+  const double inv = 1.0 / fma(a, d, -b * b);
+  const double g0 = r.f0[0], g1 = r.f1[0];
+  r.f0[0] = (d * g0 - b * g1) * inv;
+  r.f1[0] = (a * g1 - b * g0) * inv;
+}
+
+constexpr int kArMaxCtas = 8;
+constexpr size_t kArSmem = 214 * 1024;  // for the arrays of one CTA
+
+// K = cluster.num_blocks() CTAs; base: the store of each CTA's CrArrays;
+// top: kCrArrays x kArMaxCtas doubles (CTA 0's are used); next_x: the next
+// CTA's first solution.
+__device__ void cr_solve(const cg::cluster_group& cl, double* base, double* top, double* next_x,
+                         int mk, const double* w, const double* y, int n, double lam) {
+  const int K = (int)cl.num_blocks(), rank = (int)cl.block_rank(), row0 = rank * mk;
+  const CrArrays r(base, mk);
+  for (int l = threadIdx.x; l < mk; l += blockDim.x) {
+    const int r0 = 2 * (row0 + l), r1 = r0 + 1;
     const bool v0 = r0 < n, v1 = r1 < n;
-    r.aa[i] = v0 ? w[r0] + lam * dtd0(r0, n) : 1.0;
-    r.ab[i] = v1 ? lam * dtd1(r0, n) : 0.0;
-    r.ad[i] = v1 ? w[r1] + lam * dtd0(r1, n) : 1.0;
-    r.c00[i] = r0 + 2 < n ? lam : 0.0;                 // (r0, r0 + 2)
-    r.c01[i] = 0.0;                                     // (r0, r0 + 3)
-    r.c10[i] = r1 + 1 < n ? lam * dtd1(r1, n) : 0.0;    // (r1, r1 + 1)
-    r.c11[i] = r1 + 2 < n ? lam : 0.0;                  // (r1, r1 + 2)
-    r.f0[i] = v0 ? w[r0] * y[r0] : 0.0;
-    r.f1[i] = v1 ? w[r1] * y[r1] : 0.0;
+    r.aa[l] = v0 ? w[r0] + lam * dtd0(r0, n) : 1.0;
+    r.ab[l] = v1 ? lam * dtd1(r0, n) : 0.0;
+    r.ad[l] = v1 ? w[r1] + lam * dtd0(r1, n) : 1.0;
+    r.c00[l] = r0 + 2 < n ? lam : 0.0;                 // (r0, r0 + 2)
+    r.c01[l] = 0.0;                                     // (r0, r0 + 3)
+    r.c10[l] = r1 + 1 < n ? lam * dtd1(r1, n) : 0.0;    // (r1, r1 + 1)
+    r.c11[l] = r1 + 2 < n ? lam : 0.0;                  // (r1, r1 + 2)
+    r.f0[l] = v0 ? w[r0] * y[r0] : 0.0;
+    r.f1[l] = v1 ? w[r1] * y[r1] : 0.0;
   }
   __syncthreads();
-  for (int s = 1; s < m; s *= 2) {
-    // rows leaving at this level: invert A_j, keep their left coupling
-    for (int j = s + 2 * s * threadIdx.x; j < m; j += 2 * s * blockDim.x) {
-      const double a = r.aa[j], b = r.ab[j], d = r.ad[j];
-      const double inv = 1.0 / fma(a, d, -b * b);
-      r.aa[j] = d * inv;
-      r.ab[j] = -b * inv;
-      r.ad[j] = a * inv;
-      const M2 L = tr(r.C(j - s));
-      r.l00[j] = L.a;
-      r.l01[j] = L.b;
-      r.l10[j] = L.c;
-      r.l11[j] = L.d;
-    }
-    __syncthreads();
-    // rows staying: take in both neighbours
-    for (int i = 2 * s * threadIdx.x; i < m; i += 2 * s * blockDim.x) {
-      M2 Ai = r.A(i);
-      double g0 = r.f0[i], g1 = r.f1[i];
-      if (i >= s) {
-        const int j = i - s;
-        const M2 Cj = r.C(j);
-        M2 al = mm(tr(Cj), r.A(j));
-        al = {-al.a, -al.b, -al.c, -al.d};
-        const M2 t = mm(al, Cj);
-        Ai = {Ai.a + t.a, Ai.b + t.b, Ai.c + t.c, Ai.d + t.d};
-        g0 = fma(al.a, r.f0[j], fma(al.b, r.f1[j], g0));
-        g1 = fma(al.c, r.f0[j], fma(al.d, r.f1[j], g1));
-      }
-      M2 Cn = {0.0, 0.0, 0.0, 0.0};
-      if (i + s < m) {
-        const int j = i + s;
-        const M2 Ci = r.C(i);
-        M2 ga = mm(Ci, r.A(j));
-        ga = {-ga.a, -ga.b, -ga.c, -ga.d};
-        const M2 t = mm(ga, tr(Ci));
-        Ai = {Ai.a + t.a, Ai.b + t.b, Ai.c + t.c, Ai.d + t.d};
-        g0 = fma(ga.a, r.f0[j], fma(ga.b, r.f1[j], g0));
-        g1 = fma(ga.c, r.f0[j], fma(ga.d, r.f1[j], g1));
-        Cn = mm(ga, r.C(j));
-      }
-      r.aa[i] = Ai.a;
-      r.ab[i] = 0.5 * (Ai.b + Ai.c);
-      r.ad[i] = Ai.d;
-      r.c00[i] = Cn.a;
-      r.c01[i] = Cn.b;
-      r.c10[i] = Cn.c;
-      r.c11[i] = Cn.d;
-      r.f0[i] = g0;
-      r.f1[i] = g1;
+  // the CTA before: its rows are read while they are the leaving ones, which
+  // nothing changes until the solution comes back
+  const CrArrays rp(K > 1 && rank > 0 ? cl.map_shared_rank(base, rank - 1) : base, mk);
+  auto sync = [&]() {
+    if (K > 1) cl.sync();
+    else __syncthreads();
+  };
+  for (int s = 1; s < mk; s *= 2) {
+    for (int j = s + 2 * s * threadIdx.x; j < mk; j += 2 * s * blockDim.x) cr_leave(r, j, r.C(j - s));
+    sync();
+    for (int i = 2 * s * threadIdx.x; i < mk; i += 2 * s * blockDim.x) {
+      if (i > 0) cr_stay(r, i, r, i - s, i + s);
+      else cr_stay(r, i, rp, rank > 0 ? mk - s : -1, i + s);
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    const double a = r.aa[0], b = r.ab[0], d = r.ad[0];
-    const double inv = 1.0 / fma(a, d, -b * b);
-    const double g0 = r.f0[0], g1 = r.f1[0];
-    r.f0[0] = (d * g0 - b * g1) * inv;
-    r.f1[0] = (a * g1 - b * g0) * inv;
-  }
-  __syncthreads();
-  for (int s = m / 2; s >= 1; s /= 2) {
-    for (int j = s + 2 * s * threadIdx.x; j < m; j += 2 * s * blockDim.x) {
-      const double x0 = r.f0[j - s], x1 = r.f1[j - s];
-      double g0 = r.f0[j] - fma(r.l00[j], x0, r.l01[j] * x1);
-      double g1 = r.f1[j] - fma(r.l10[j], x0, r.l11[j] * x1);
-      if (j + s < m) {
-        const double y0 = r.f0[j + s], y1 = r.f1[j + s];
-        g0 -= fma(r.c00[j], y0, r.c01[j] * y1);
-        g1 -= fma(r.c10[j], y0, r.c11[j] * y1);
+  if (K == 1) {
+    if (threadIdx.x == 0) cr_last(r);
+    __syncthreads();
+  } else {
+    // CTA 0 gathers the K rows left, reduces and solves them
+    cl.sync();
+    if (rank == 0) {
+      const CrArrays t(top, kArMaxCtas);
+      if (threadIdx.x < (unsigned)K) {
+        const CrArrays q(cl.map_shared_rank(base, threadIdx.x), mk);
+        const int l = threadIdx.x;
+        t.aa[l] = q.aa[0];
+        t.ab[l] = q.ab[0];
+        t.ad[l] = q.ad[0];
+        t.c00[l] = q.c00[0];
+        t.c01[l] = q.c01[0];
+        t.c10[l] = q.c10[0];
+        t.c11[l] = q.c11[0];
+        t.f0[l] = q.f0[0];
+        t.f1[l] = q.f1[0];
       }
-      r.f0[j] = fma(r.aa[j], g0, r.ab[j] * g1);
-      r.f1[j] = fma(r.ab[j], g0, r.ad[j] * g1);
+      __syncthreads();
+      for (int s = 1; s < K; s *= 2) {
+        const int j = s + 2 * s * threadIdx.x, i = 2 * s * threadIdx.x;
+        if (j < K) cr_leave(t, j, t.C(j - s));
+        __syncthreads();
+        if (i < K) cr_stay(t, i, t, i - s, i + s < K ? i + s : -1);
+        __syncthreads();
+      }
+      if (threadIdx.x == 0) cr_last(t);
+      __syncthreads();
+      for (int s = K / 2; s >= 1; s /= 2) {
+        const int j = s + 2 * s * threadIdx.x;
+        if (j < K) cr_back(t, j, s, K, 0.0, 0.0);
+        __syncthreads();
+      }
     }
+    cl.sync();
+    if (threadIdx.x < 2) {  // this CTA's first solution and the next one's
+      const CrArrays t(cl.map_shared_rank(top, 0), kArMaxCtas);
+      const double* f = threadIdx.x == 0 ? t.f0 : t.f1;
+      (threadIdx.x == 0 ? r.f0 : r.f1)[0] = f[rank];
+      next_x[threadIdx.x] = rank + 1 < K ? f[rank + 1] : 0.0;
+    }
+    __syncthreads();
+  }
+  const double y0 = K > 1 ? next_x[0] : 0.0, y1 = K > 1 ? next_x[1] : 0.0;
+  for (int s = mk / 2; s >= 1; s /= 2) {
+    for (int j = s + 2 * s * threadIdx.x; j < mk; j += 2 * s * blockDim.x)
+      cr_back(r, j, s, mk, y0, y1);
     __syncthreads();
   }
 }
@@ -197,67 +300,99 @@ struct ArplsArgs {
   double lam, ratio;
 };
 
-// One CTA per spectrum: the weighted solves by block cyclic reduction,
-// the residual statistics and the reweighting, all parallel over the CTA.
+// One cluster of K CTAs per spectrum (K = 1: one CTA): the weighted solves by
+// block cyclic reduction, the residual statistics and the reweighting, all
+// parallel over the cluster. FP64 issue bounds it (two lanes per cycle and
+// SM on GB300; a solve and reweighting of 4096 channels is about 4e5
+// operations) and the levels' latency.
 __global__ void __launch_bounds__(kArThreads, 1) arpls_kernel(ArplsArgs g) {
   extern __shared__ double ar_sm[];
-  __shared__ double red[kArWarps];
-  const int sys = blockIdx.x, n = g.n, m = cr_rows(n);
+  __shared__ double red[kArWarps + 1][2];
+  __shared__ double top[kCrArrays * kArMaxCtas];
+  __shared__ double next_x[2];
+  __shared__ double parts[2][kArMaxCtas][2];
+  const cg::cluster_group cl = cg::this_cluster();
+  const int K = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int sys = blockIdx.x / K, n = g.n, mk = cr_rows(n) / K;
   double* w = g.work + (size_t)sys * 2 * n;
   double* wt = w + n;
-  double* cr = g.in_smem ? ar_sm
-                         : g.work + (size_t)g.n_sys * 2 * n + (size_t)sys * kCrArrays * m;
-  const CrArrays r(cr, m);
+  double* base = g.in_smem ? ar_sm
+                           : g.work + (size_t)g.n_sys * 2 * n + (size_t)sys * kCrArrays * mk;
+  const CrArrays r(base, mk);
   const double* y = g.y + (size_t)sys * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) w[i] = 1.0;
+  // this CTA's channels
+  const int i0 = 2 * rank * mk, i1 = min(n, i0 + 2 * mk);
+  auto z = [&](int i) { return (i & 1) ? r.f1[(i - i0) >> 1] : r.f0[(i - i0) >> 1]; };
+  // sums of two values over the cluster, in a fixed order
+  int buf = 0;
+  auto sum2 = [&](double& a, double& b) {
+    block_sum2(a, b, red);
+    if (K == 1) return;
+    if (threadIdx.x < (unsigned)K) {
+      double* dst = cl.map_shared_rank(&parts[buf][rank][0], threadIdx.x);
+      dst[0] = a;
+      dst[1] = b;
+    }
+    cl.sync();
+    if (threadIdx.x < 2) {  // two threads: FP64 issue is scarce
+      double t = 0.0;
+      for (int c = 0; c < K; ++c) t += parts[buf][c][threadIdx.x];
+      red[kArWarps][threadIdx.x] = t;
+    }
+    __syncthreads();
+    a = red[kArWarps][0];
+    b = red[kArWarps][1];
+    buf ^= 1;  // the other buffer's readers passed this barrier
+  };
+  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) w[i] = 1.0;
   __syncthreads();
   int solves = 0;
+  double w2 = (double)n;  // sum of the squared weights
   while (solves < g.itermax) {
-    cr_solve(r, m, w, y, n, g.lam);
+    cr_solve(cl, base, top, next_x, mk, w, y, n, g.lam);
     ++solves;
-    // z_i is f0 / f1 of block row i / 2
     double sn = 0.0, cn = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double d = y[i] - ((i & 1) ? r.f1[i >> 1] : r.f0[i >> 1]);
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+      const double d = y[i] - z(i);
       if (d < 0.0) {
         sn += d;
         cn += 1.0;
       }
     }
-    sn = block_sum(sn, red);
-    cn = block_sum(cn, red);
+    sum2(sn, cn);
     if (cn == 0.0) break;
     const double mneg = sn / cn;
-    double s2 = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double d = y[i] - ((i & 1) ? r.f1[i >> 1] : r.f0[i >> 1]);
+    double s2 = 0.0, unused = 0.0;
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+      const double d = y[i] - z(i);
       if (d < 0.0) s2 += (d - mneg) * (d - mneg);
     }
-    const double sd = sqrt(block_sum(s2, red) / cn);
+    sum2(s2, unused);
+    const double sd = sqrt(s2 / cn);
     if (!(sd > 0.0)) break;
-    const double thr = 2.0 * sd - mneg;
-    double dw2 = 0.0, w2 = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double d = y[i] - ((i & 1) ? r.f1[i >> 1] : r.f0[i >> 1]);
-      const double wn = 1.0 / (1.0 + exp(2.0 * (d - thr) / sd));
+    const double thr = 2.0 * sd - mneg, scale = 2.0 / sd;
+    double dw2 = 0.0, wn2 = 0.0;
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+      const double d = y[i] - z(i);
+      const double wn = 1.0 / (1.0 + exp((d - thr) * scale));
       dw2 += (w[i] - wn) * (w[i] - wn);
-      w2 += w[i] * w[i];
+      wn2 += wn * wn;
       wt[i] = wn;
     }
-    dw2 = block_sum(dw2, red);
-    w2 = block_sum(w2, red);
+    sum2(dw2, wn2);
     if (sqrt(dw2) / sqrt(w2) < g.ratio) break;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) w[i] = wt[i];
+    w2 = wn2;
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) w[i] = wt[i];
     __syncthreads();
   }
   __syncthreads();
-  double* z = g.z + (size_t)sys * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double zi = (i & 1) ? r.f1[i >> 1] : r.f0[i >> 1];
-    z[i] = zi;
+  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    const double zi = z(i);
+    g.z[(size_t)sys * n + i] = zi;
     if (g.zf) g.zf[(size_t)sys * n + i] = (float)zi;
   }
-  if (threadIdx.x == 0 && g.iters) g.iters[sys] = solves;
+  if (rank == 0 && threadIdx.x == 0 && g.iters) g.iters[sys] = solves;
+  if (K > 1) cl.sync();  // no CTA leaves while another may read its rows
 }
 
 // y[(I * N + a) * n_chan + j]: mean of beam a, channel j over interval I,
@@ -328,15 +463,28 @@ __global__ void ccm_bandpass_kernel(const int64_t* __restrict__ sums, int64_t n_
 
 }  // namespace
 
-size_t arpls_smem_bytes(int n) {
-  const size_t b = (size_t)kCrArrays * cr_rows(n) * sizeof(double);
-  return b <= 214 * 1024 ? b : 0;  // 0: the arrays live in global memory
+// CTAs per spectrum: two for long spectra that leave SMs idle, and as many as
+// it takes for the arrays to fit shared memory. Measured on GB300, us a call
+// of 5 to 6 solves with 1 / 2 / 4 / 8 CTAs: 38 spectra of 4096 channels 904 /
+// 696 / 994 / 1290, 190 spectra 1650 / 1845 / 2793 / 5303, 38 spectra of 1000
+// channels 420 / 431 / 649 / 1093 (the cluster's barriers and the serial top
+// outweigh the share of the FP64 work).
+int arpls_ctas(int n, int n_sys, int sm_count) {
+  const int m = cr_rows(n);
+  int k = m >= 1024 && (int64_t)n_sys * 2 <= sm_count ? 2 : 1;
+  while (k < kArMaxCtas && (size_t)kCrArrays * (m / k) * sizeof(double) > kArSmem) k *= 2;
+  return k;
+}
+// Shared memory of one of k CTAs; 0: the arrays live in global memory (k = 1)
+size_t arpls_smem_bytes(int n, int k) {
+  const size_t b = (size_t)kCrArrays * (cr_rows(n) / k) * sizeof(double);
+  return b <= kArSmem ? b : 0;
 }
 
 size_t arpls_work_doubles(int n, int n_sys) {
   // the weights always; the reduction arrays when they are not in shared memory
   return (size_t)2 * n * n_sys +
-         (arpls_smem_bytes(n) ? 0 : (size_t)kCrArrays * cr_rows(n) * n_sys);
+         (arpls_smem_bytes(n, kArMaxCtas) ? 0 : (size_t)kCrArrays * cr_rows(n) * n_sys);
 }
 
 cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, int n, double lam,
@@ -355,13 +503,24 @@ cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, i
   g.itermax = itermax;
   g.lam = lam;
   g.ratio = ratio;
-  const size_t smem = arpls_smem_bytes(n);
+  int k = arpls_ctas(n, n_sys, pl->sm_count);
+  const size_t smem = arpls_smem_bytes(n, k);
+  if (!smem) k = 1;  // one CTA per spectrum on global memory
   g.in_smem = smem ? 1 : 0;
   cudaError_t e = cudaFuncSetAttribute(arpls_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  arpls_kernel<<<n_sys, kArThreads, smem, pl->stream>>>(g);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)n_sys * k);
+  cfg.blockDim = dim3(kArThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = pl->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {(unsigned)k, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, arpls_kernel, g);
 }
 
 cudaError_t launch_bandpass_input(const mraid_plan_s* pl, const int64_t* d_sums, int interval, double* d_y) {
