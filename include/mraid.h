@@ -285,9 +285,9 @@ mraid_status mraid_run_bandpass(mraid_plan_t plan, const void* d_data,
 
 /* Autotuner (the paper has no counterpart; it picks among this library's
  * kernel variants). Times, `reps` runs each on d_data, every Gram variant
- * that fits the plan's shape (for 8-bit samples and up to 23 beams ten ids:
- * even ones choose the channels per work item by the shape, odd ones take 64;
- * and the CUDA-core Gram) and the register
+ * that fits the plan's shape (for 8-bit samples and up to 39 beams ten ids:
+ * even ones choose the channels per work item by the shape, odd ones take 64
+ * for up to 23 beams; and the CUDA-core Gram) and the register
  * eigensolvers (Jacobi rounds in a loop; the Jacobi sweep unrolled;
  * Householder tridiagonalisation + implicit QR in two code layouts), and
  * keeps the fastest of each for this plan. *gram_choice: -1 = CUDA-core,
@@ -300,7 +300,7 @@ mraid_status mraid_autotune(mraid_plan_t plan, const void* d_data, int32_t reps,
 /* Select variants by id (e.g. from a tuning cache). Gram: -1 = CUDA-core,
  * 0..9 tensor-core Gram: for up to 23 beams even ids choose the channels per
  * work item by the shape and odd ids take 64; for 24..127 beams any id >= 0
- * selects the large-beam tensor-core Gram (exact in pieces of <= 1024
+ * selects the tensor-core Gram of that beam count (exact in pieces of <= 1024
  * samples).
  * Eigensolver (beam counts with a one-thread-per-matrix kernel: 2, 3, 4, 13,
  * 19; other counts always use the warp-per-matrix Jacobi): 0 = Jacobi,

@@ -1,44 +1,53 @@
-// gram_mma.cu - exact augmented Gram sums of 8-bit multi-beam data for 2..23
+// gram_mma.cu - exact augmented Gram sums of 8-bit multi-beam data for 2..39
 // beams, fused with the correlation.
 //
 // Section 3.2, Eq. 1. For a cell (channel j, sub-integration k) with samples
 // x_b(t), the kernel forms G = Y Y^T with Y = [x - 128; 1]. The centred
 // values are exact in f16, products are integers of magnitude <= 2^14 and
 // sums over <= 1024 samples are integers of magnitude <= 2^24, so FP32
-// accumulation is exact; longer sub-integrations are flushed as int64 every
-// 1024 samples. cov_ab = n G_ab - G_a G_b is exact in int64 and
+// accumulation is exact; longer sub-integrations are added up every 1024
+// samples, as int32 in shared memory for up to 127 such pieces and as int64
+// in the sums beyond that. cov_ab = n G_ab - G_a G_b is exact in int64 and
 // r_ab = cov_ab / sqrt(var_a var_b) is rounded to float once. The raw sums
 // are S_ab = G_ab + 128 (G_a + G_b) + 128^2 n and S_a = G_a + 128 n.
 //
-// Why register fragments (mma.sync) and not tcgen05: a cell's Gram is 24 x 24
+// Why register fragments (mma.sync) and not tcgen05: a cell's Gram is 40 x 40
 // at most, and the samples lie channel by channel in memory. A 128-row
 // tcgen05 tile of 16 beams x 8 channels keeps 1/8 of its products, and its
 // operands cross shared memory 5 times as f16; that kernel was bound by
-// shared memory at 3.4 TB/s of samples. Here a warp owns 8 channels and every
-// product is of one channel: a lane reads 8 bytes (8 channels) of one beam
+// shared memory at 3.4 TB/s of samples. Here a warp owns 8 channels (4 from 24 beams on) and every
+// product is of one channel: a lane reads the warp's channels of one beam
 // and one sample, a pair of samples becomes an f16x2 register by byte
 // permutes (x in the low mantissa bits of 1024, minus 1152), and that
 // register is at once an A and a B fragment of its channel's Gram, because
 // the order of the samples within K is free. Products per channel and 16
-// samples: block rows (0, 1) x every block column, and the last block of an
-// odd count by itself.
+// samples: each pair of 8-beam block rows x the block columns from its first
+// on, and the last block of an odd count by itself.
 //
 // Layout: a work item is one sub-integration x 32, 64, 96 or 128 channels
-// (4, 8, 12 or 16 warps, as many as the accumulators leave registers for);
+// (4, 8, 12 or 16 warps, as many as the accumulators leave registers for; 32
+// channels and 8 warps from 24 beams on);
 // stages of 16 samples x all beams come by TMA with a swizzle under which a
 // warp's 8-byte loads meet two-way conflicts at most, into a ring as deep as
-// shared memory allows; the warps take turns to issue the copies. Rows of 64
-// bytes and more on their own multiples matter: 16- and 32-byte rows stream
+// shared memory allows; the warps take turns to issue the copies. Wide rows
+// on their own multiples matter: 16- and 32-byte rows stream
 // at 4.7-4.8 TB/s on GB300, 64-byte ones at 6.3-6.7, 128-byte ones at 7.1.
 // Layouts that no tensor map takes (odd channel counts, misaligned buffers)
-// fill the same ring by cp.async or byte loads.
+// fill the same ring by cp.async, or at odd addresses from pairs of aligned
+// words (byte by byte, 36 beams x 1001 channels x 1000 samples x 20 took 4.4
+// ms, so 1.96).
 //
 // Measured on GB300 (50 sub-integrations x 4096 channels x 1024 samples):
 // 19 beams 0.89 ms (4.5 TB/s of samples; the tcgen05 kernel 1.20 ms), 13
 // beams 0.54 ms (0.91), 7 beams 0.35 ms (0.84); with 128 samples per
 // sub-integration, where the epilogue weighs most, 1.70, 0.98 and 0.63 ms
 // (6.27, 4.64 and 4.21). 1000 channels x 1000 samples x 40 (no tensor map)
-// 0.38 ms, on dp4a 0.62 ms. Without its copies the 19-beam kernel takes 0.75
+// 0.38 ms, on dp4a 0.62 ms. With more than 1024 samples and from 24 beams on,
+// correlation included: 36 beams x 2048 channels x 2048 samples x 38 1.58 ms
+// (tcgen05 with two channels per 128-row tile 3.52 + 0.17), 24 beams x 4096 x
+// 1024 x 20 0.66 ms (1.27 + 0.09), 39 beams x 2048 x 1024 x 38 0.87 ms (1.82
+// + 0.22); at 40 beams the accumulators of four channels would no longer fit
+// a warp's registers. Without its copies the 19-beam kernel takes 0.75
 // ms, without its products 0.8: bound by both, the permutes' and MMAs' issue
 // at 3 warps per scheduler and the copies that pause in the epilogue.
 //
@@ -49,6 +58,7 @@
 #include <stdint.h>
 
 #include <type_traits>
+#include <utility>
 
 #include "internal.h"
 #include "tc_ptx.h"
@@ -56,38 +66,52 @@
 namespace mraid {
 namespace {
 
-constexpr int kCW = 8;                       // channels per warp
 constexpr int kMmLag = 1;  // stages between a slot's last read and its refill
 constexpr int kMmT = 16;                     // samples per stage: one K step
 constexpr int kMmMaxD = 12;                  // ring depth bound
 constexpr int kMmPiece = 1024;               // samples accumulated before a flush
+constexpr int kMmLongMax = kMmPieceMax;      // samples whose int32 sums cannot overflow (127 pieces)
 constexpr size_t kMmSmem = 226 * 1024;
 constexpr int kMmEpi = 2;                    // channels staged at a time by the epilogue
 
 // NB 8-beam blocks; kHalf: the last one holds at most four slots, and its
 // fragment carries them for two channels (lanes of rows 0..3 the even one,
 // 4..7 the odd one); A_, B_: channels of a stage's two boxes (B_ 0: one box).
-template <int NB_, bool kHalf_, int A_, int B_>
+// kLong_: sub-integrations of several pieces, added as int32 in shared memory.
+template <int NB_, bool kHalf_, int A_, int B_, int CW_ = 8, bool kLong_ = false>
 struct MmCfg {
+  static constexpr bool kLong = kLong_;
+  static constexpr int kCW = CW_;  // channels per warp
   static constexpr int NB = NB_, kChA = A_, kChB = B_, kCh = A_ + B_;
   static constexpr bool kHalf = kHalf_;
   static constexpr int kWarps = kCh / kCW, kThreads = 32 * kWarps;
   static constexpr int kTile = kMmT * kCh;  // bytes of one beam in a stage
-  // floats of one channel's products in the epilogue
-  static constexpr int kG = NB == 1 ? 64 : (NB == 2 ? 192 : (kHalf ? 272 : 384));
+  // One channel's products in the epilogue, in floats: per block row pair
+  // (2p, 2p + 1) the 8 x 8 of the diagonal block 2p, then 16 x 8 for every
+  // later block column; the last block of an odd count by itself.
+  __host__ __device__ static constexpr int pair_at(int p) {
+    int at = 0;
+    for (int q = 0; q < p; ++q) at += 64 + 128 * (NB - 1 - 2 * q);
+    return at;
+  }
+  static constexpr int kG = kHalf ? 272 : pair_at(NB / 2) + (NB & 1 ? 64 : 0);
+  using Sum = typename std::conditional<kLong, int32_t, float>::type;
   struct Shared {
     uint64_t full[kMmMaxD], empty[kMmMaxD];
     uint32_t lut[(8 * NB) * (8 * NB + 1) / 2];  // G offset | a << 16 | b << 24
-    alignas(16) float g[kWarps][kMmEpi][kG];
+    // a group of channels' products; of several pieces, every channel's sums
+    alignas(16) Sum g[kWarps][kLong ? kCW : kMmEpi][kG];
     int2 row[kWarps][kMmEpi][8 * NB];  // per beam: sum of the centred samples, 1/sqrt(var)
   };
   // Where the pair (a, b), a <= b, lies in a channel's products.
   __host__ __device__ static constexpr int off(int a, int b) {
     const int ba = a >> 3, bb = b >> 3, e = (a & 7) * 8 + (b & 7);
-    if (bb == 0) return e;
-    if (bb == 1) return 64 + a * 8 + (b & 7);
-    if (kHalf) return ba < 2 ? 192 + a * 4 + (b & 7) : 256 + (a & 7) * 4 + (b & 7);
-    return ba < 2 ? 192 + a * 8 + (b & 7) : 320 + e;
+    if (kHalf && bb == 2)
+      return ba < 2 ? 192 + a * 4 + (b & 7) : 256 + (a & 7) * 4 + (b & 7);
+    int at = 0;
+    for (int q = 0; q < ba / 2; ++q) at += 64 + 128 * (NB - 1 - 2 * q);
+    if (bb == (ba & ~1)) return at + e;
+    return at + 64 + (bb - (ba & ~1) - 1) * 128 + (ba & 1) * 64 + e;
   }
   static constexpr size_t kFixed = 1024 + sizeof(Shared);
   static constexpr int stage_bytes(int n_beam) { return (n_beam + 2) * kTile; }
@@ -100,7 +124,8 @@ struct MmCfg {
 struct MmArgs {
   const uint8_t* data;  // plain copies: the samples, beams beam_stride apart
   int64_t beam_stride;
-  int vec;  // plain copies: bytes per copy (8 or 4: cp.async; 1: byte loads)
+  const uint8_t* data_end;  // one past the last sample
+  int vec;  // plain copies: bytes per copy (8 or 4: cp.async; 1: any address)
   int n_beam, n_chan, n_samp_sub, sub0, n_sub;
   int depth;  // ring stages
   int64_t* sums;
@@ -129,6 +154,12 @@ __device__ __forceinline__ float i64_to_float(int64_t x) {
               __uint_as_float(0x4b000000u | lo) - 8388608.f);
 }
 
+template <bool kLong>
+__device__ __forceinline__ float cov_to_float(int64_t x) {
+  if constexpr (kLong) return (float)x;  // beyond the two mantissas
+  else return i64_to_float(x);
+}
+
 __device__ __forceinline__ uint32_t f16_sub(uint32_t x, uint32_t y) {
   uint32_t r;
   asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
@@ -136,10 +167,22 @@ __device__ __forceinline__ uint32_t f16_sub(uint32_t x, uint32_t y) {
 }
 
 template <int kImm>
-__device__ __forceinline__ uint2 lds64(uint32_t addr) {
-  uint2 v;
+__device__ __forceinline__ void lds_word(uint32_t addr, uint2& v) {
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2+%3];" : "=r"(v.x), "=r"(v.y) : "r"(addr), "n"(kImm));
-  return v;
+}
+template <int kImm>
+__device__ __forceinline__ void lds_word(uint32_t addr, uint1& v) {
+  asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v.x) : "r"(addr), "n"(kImm));
+}
+__device__ __forceinline__ uint32_t word(const uint2& v, int q) { return q ? v.y : v.x; }
+__device__ __forceinline__ uint32_t word(const uint1& v, int) { return v.x; }
+template <class F, int... I>
+__device__ __forceinline__ void static_loop_(F&& f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+template <int K, class F>
+__device__ __forceinline__ void static_loop(F&& f) {  // f(constant 0 .. K - 1)
+  static_loop_(f, std::make_integer_sequence<int, K>{});
 }
 // A lane constant that the compiler keeps instead of computing it again.
 __device__ __forceinline__ void pin(uint32_t& x) { asm volatile("" : "+r"(x)); }
@@ -220,7 +263,9 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       tma_load_3d(dst + box_a, &map_b, ch0 + C::kChA, t0, 0, &s->full[slot]);
   };
   // the same by every thread's own copies, for layouts that no tensor map
-  // takes; a thread fills one place of every beam (or of every other one)
+  // takes; a thread fills one place of every beam (or of every other one),
+  // worked out anew each time: kept in registers it made few beams 15 %
+  // faster but 19 beams x 1000 x 1000 x 40 0.52 ms instead of 0.38 (spills)
   int f_it = blockIdx.x, f_st = 0, f_slot = 0;  // next stage to fill
   auto fill = [&](int r) {
     const int v = g.vec, words = v == 8 ? C::kCh / 8 : C::kCh / 4;
@@ -240,15 +285,40 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       for (int b = 0; b < N; ++b)
         if (mine) copy_async<4>(dst + b * kMmT * pitch, src + b * g.beam_stride);
     } else if (mine) {
-      const int nc = min(4, g.n_chan - ch);
+      const int nc = g.n_chan - ch;
+      // four bytes at any address: of the two aligned words about them, where
+      // the first and the last beam's lie within the samples (one branch for
+      // all beams, so that eight beams' loads are in flight)
+      auto word = [](const uint8_t* p) { return p - (reinterpret_cast<uintptr_t>(p) & 3); };
+      if (nc >= 4 && word(src) >= g.data &&
+          word(src + (N - 1) * g.beam_stride) + 8 <= g.data_end) {
+        for (int b0 = 0; b0 < N; b0 += 8) {
+          uint32_t lo[8], hi[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint8_t* p = src + min(b0 + j, N - 1) * g.beam_stride;
+            const uint32_t* w = reinterpret_cast<const uint32_t*>(word(p));
+            lo[j] = __ldg(w);
+            hi[j] = __ldg(w + 1);
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int b = min(b0 + j, N - 1);
+            const uint32_t at = (uint32_t)reinterpret_cast<uintptr_t>(src + b * g.beam_stride) & 3;
+            const uint32_t x = __funnelshift_r(lo[j], hi[j], at * 8);
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + b * kMmT * pitch), "r"(x) : "memory");
+          }
+        }
+      } else {
 #pragma unroll 4
-      for (int b = 0; b < N; ++b) {
-        const uint8_t* p = src + b * g.beam_stride;
-        uint32_t x = p[0];
-        if (nc > 1) x |= (uint32_t)p[1] << 8;
-        if (nc > 2) x |= (uint32_t)p[2] << 16;
-        if (nc > 3) x |= (uint32_t)p[3] << 24;
-        asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + b * kMmT * pitch), "r"(x) : "memory");
+        for (int b = 0; b < N; ++b) {
+          const uint8_t* p = src + b * g.beam_stride;
+          uint32_t x = p[0];
+          if (nc > 1) x |= (uint32_t)p[1] << 8;
+          if (nc > 2) x |= (uint32_t)p[2] << 16;
+          if (nc > 3) x |= (uint32_t)p[3] << 24;
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + b * kMmT * pitch), "r"(x) : "memory");
+        }
       }
     }
     if (!(blockIdx.x == 0 && r == g.withhold)) {
@@ -275,11 +345,13 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   // every 4; odd beams read the two halves of an 8-sample group in the
   // opposite order (their pairs are put back by the permute selectors)
   const int g8 = lane >> 2, t = lane & 3, odd = g8 & 1;
-  const bool in_a = warp < C::kChA / kCW;
+  const bool in_a = warp < C::kChA / C::kCW;
   const int pitch = in_a ? C::kChA : C::kChB;                       // bytes per row
-  const int wc = in_a ? warp >> 1 : (warp - C::kChA / kCW) >> 1;   // 16-byte column
-  auto place = [&](int r) {  // this warp's 8 bytes of row r, swizzled
-    return r * pitch + ((wc ^ swizzle(pitch, r)) << 4) + ((warp & 1) << 3);
+  const int wc = in_a ? warp >> 1 : (warp - C::kChA / C::kCW) >> 1;   // 16-byte column
+  const int cb = C::kCW * warp - (in_a ? 0 : C::kChA);
+  auto place = [&](int r) {  // this warp's bytes of row r, swizzled
+    if constexpr (C::kCW == 8) return r * pitch + ((wc ^ swizzle(pitch, r)) << 4) + ((warp & 1) << 3);
+    return r * pitch + (((cb >> 4) ^ swizzle(pitch, r)) << 4) + (cb & 15);
   };
   const int q0 = place(t + (odd ? 4 : 0)), q1 = place(t + (odd ? 0 : 4));
   uint32_t sel_lo = odd ? 0x1504u : 0x5140u;
@@ -300,7 +372,8 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   pin(L0);
   pin(L1);
 
-  constexpr int kAcc = kHalf || NB == 2 ? 2 : (NB == 1 ? 1 : 4);  // per channel
+  // accumulator tiles per channel
+  constexpr int kAcc = kHalf ? 2 : (NB / 2) * ((NB + 1) / 2 + 1) + (NB & 1);
   constexpr int kFull = kHalf ? NB - 1 : NB;
 
   int slot = 0;
@@ -311,23 +384,24 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   while (duty < D) duty += C::kWarps;
   bool ok = true;
   for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-    const int k = it / chunks, ch0 = it % chunks * C::kCh + kCW * warp;
+    const int k = it / chunks, ch0 = it % chunks * C::kCh + C::kCW * warp;
     for (int piece0 = 0; piece0 < stages && ok; piece0 += kMmPiece / kMmT) {
       const int piece1 = min(stages, piece0 + kMmPiece / kMmT);
-      float acc[kCW][kAcc][4];
-      float acc2[kHalf ? kCW / 2 : 1][2][4];  // of two channels: blocks (0, 1) x last, last x last
+      float acc[C::kCW][kAcc][4];
+      float acc2[kHalf ? C::kCW / 2 : 1][2][4];  // of two channels: blocks (0, 1) x last, last x last
 #pragma unroll
-      for (int c = 0; c < kCW; ++c)
+      for (int c = 0; c < C::kCW; ++c)
 #pragma unroll
         for (int m = 0; m < kAcc; ++m)
 #pragma unroll
           for (int i = 0; i < 4; ++i) acc[c][m][i] = 0.f;
 #pragma unroll
-      for (int c = 0; c < (kHalf ? kCW / 2 : 1); ++c)
+      for (int c = 0; c < (kHalf ? C::kCW / 2 : 1); ++c)
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc2[c][i / 4][i % 4] = 0.f;
       auto run = [&](auto pitch_c) {
         constexpr int kPitch = decltype(pitch_c)::value;
+        using Word = typename std::conditional<C::kCW == 8, uint2, uint1>::type;
         for (int st = piece0; st < piece1; ++st) {
           ok = mbar_wait(&s->full[slot], ph, g.error, g.wait_ns);
           ok = __all_sync(0xffffffffu, ok);
@@ -337,31 +411,26 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (nv < kMmT) {  // samples of the next sub-integration: the centre value
             for (int i = lane; i < (kMmT - nv) * N; i += 32) {
               const int r = nv + i / N, b = i % N;
-              *reinterpret_cast<uint2*>(stage + tile0 + b * kMmT * kPitch + place(r)) =
-                  make_uint2(0x80808080u, 0x80808080u);
+              Word* at = reinterpret_cast<Word*>(stage + tile0 + b * kMmT * kPitch + place(r));
+              if constexpr (C::kCW == 8) *at = make_uint2(0x80808080u, 0x80808080u);
+              else *at = make_uint1(0x80808080u);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
           }
-          uint2 w[NB][2][2];
+          Word w[NB][2][2];
           {
             const uint32_t so = (uint32_t)(slot * stage_bytes);
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
+            static_loop<NB>([&](auto bb) {
+              constexpr int b = decltype(bb)::value;
               const uint32_t p0 = b == NB - 1 ? L0 + so : A0 + so;
               const uint32_t p1 = b == NB - 1 ? L1 + so : A1 + so;
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                constexpr int kBlk = 8 * kMmT * kPitch;
-                if (b == 0 || b == NB - 1) {
-                  w[b][h][0] = h ? lds64<8 * kPitch>(p0) : lds64<0>(p0);
-                  w[b][h][1] = h ? lds64<8 * kPitch>(p1) : lds64<0>(p1);
-                } else {
-                  w[b][h][0] = h ? lds64<kBlk + 8 * kPitch>(p0) : lds64<kBlk>(p0);
-                  w[b][h][1] = h ? lds64<kBlk + 8 * kPitch>(p1) : lds64<kBlk>(p1);
-                }
-              }
-            }
+              constexpr int o = b == NB - 1 ? 0 : b * 8 * kMmT * kPitch;
+              lds_word<o>(p0, w[b][0][0]);
+              lds_word<o>(p1, w[b][0][1]);
+              lds_word<o + 8 * kPitch>(p0, w[b][1][0]);
+              lds_word<o + 8 * kPitch>(p1, w[b][1][1]);
+            });
           }
           // the stage is in registers: release it before the products
           __syncwarp();
@@ -392,15 +461,14 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             }
           }
 #pragma unroll
-          for (int q = 0; q < kCW / 4; ++q) {
+          for (int q = 0; q < C::kCW / 4; ++q) {
             // f: blocks 0.., f2: the half block, of two channels
             uint32_t f[4][kFull][2], f2[2][2];
 #pragma unroll
             for (int b = 0; b < NB; ++b)
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
-                const uint32_t x = q ? w[b][h][0].y : w[b][h][0].x;
-                const uint32_t y = q ? w[b][h][1].y : w[b][h][1].x;
+                const uint32_t x = word(w[b][h][0], q), y = word(w[b][h][1], q);
                 if (b < kFull) {
                   const uint32_t lo = __byte_perm(x, y, sel_lo), hi = __byte_perm(x, y, sel_lo + 0x2222u);
 #pragma unroll
@@ -420,18 +488,26 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               float(&d)[kAcc][4] = acc[4 * q + c];
-              if constexpr (NB >= 2) {
+              if constexpr (NB == 2 || NB == 3) {
 #pragma unroll
                 for (int z = 0; z < kFull; ++z)
                   mma16816(d[z], f[c][0][0], f[c][1][0], f[c][0][1], f[c][1][1], f[c][z][0],
                            f[c][z][1]);
+              } else {
+                int m = 0;
+#pragma unroll
+                for (int p = 0; p < NB / 2; ++p)
+#pragma unroll
+                  for (int z = 2 * p; z < kFull; ++z, ++m)
+                    mma16816(d[m], f[c][2 * p][0], f[c][2 * p + 1][0], f[c][2 * p][1],
+                             f[c][2 * p + 1][1], f[c][z][0], f[c][z][1]);
               }
               if constexpr (kHalf) {
                 // the other channel's columns are zero here, so both add into one tile
                 const uint32_t mk = c & 1 ? ~mask_even : mask_even;
                 mma16816(acc2[2 * q + c / 2][0], f[c][0][0], f[c][1][0], f[c][0][1],
                          f[c][1][1], f2[c / 2][0] & mk, f2[c / 2][1] & mk);
-              } else if constexpr (NB != 2) {
+              } else if constexpr (NB & 1) {
                 constexpr int L = NB - 1;
                 const int p = c & ~1;
                 mma16816(d[kAcc - 1], f[p][L][0], f[p + 1][L][0], f[p][L][1], f[p + 1][L][1],
@@ -453,23 +529,71 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       if (!ok) break;
       if (ch0 >= g.n_chan) continue;
       // ---- epilogue: a few channels at a time through the warp's staging area
-      const int n = min(g.n_samp_sub - piece0 * kMmT, kMmPiece);
+      const int n = C::kLong ? g.n_samp_sub : min(g.n_samp_sub - piece0 * kMmT, kMmPiece);
+      // channel c's accumulators into sg, or (several pieces) added to it
+      auto stage_out = [&](auto cc, typename C::Sum* sg) {
+        constexpr int c = decltype(cc)::value;
+        auto put = [&](int at, const float* d) {
+          if constexpr (C::kLong) {
+            int2* p = reinterpret_cast<int2*>(sg + at);
+            int2 v = make_int2(__float2int_rn(d[0]), __float2int_rn(d[1]));
+            if (piece0 > 0) {
+              v.x += p->x;
+              v.y += p->y;
+            }
+            *p = v;
+          } else {
+            *reinterpret_cast<float2*>(sg + at) = make_float2(d[0], d[1]);
+          }
+        };
+        const int e = g8 * 8 + 2 * t;
+        int m = 0;
+#pragma unroll
+        for (int p = 0; p < NB / 2; ++p) {
+          const int at = C::pair_at(p) + e;
+#pragma unroll
+          for (int z = 2 * p; z < kFull; ++z, ++m) {
+            if (z == 2 * p) {
+              put(at, acc[c][m]);  // the other half is block (2p, 2p + 1) again
+            } else {
+              put(at + 64 + 128 * (z - 2 * p - 1), acc[c][m]);
+              put(at + 128 + 128 * (z - 2 * p - 1), acc[c][m] + 2);
+            }
+          }
+        }
+        if constexpr (!kHalf && (NB & 1)) put(C::kG - 64 + e, acc[c][kAcc - 1] + 2 * (c & 1));
+        if constexpr (kHalf) {
+          if ((t >> 1) == (c & 1)) {  // this channel's four of the eight columns
+            const int e4 = g8 * 4 + 2 * (t & 1);
+            put(192 + e4, acc2[c / 2][0]);
+            put(224 + e4, acc2[c / 2][0] + 2);
+            if ((g8 >> 2) == (c & 1))
+              put(256 + (g8 & 3) * 4 + 2 * (t & 1), acc2[c / 2][1] + ((c / 2) & 1 ? 2 : 0));
+          }
+        }
+      };
+      if constexpr (C::kLong) {
+        static_loop<C::kCW>([&](auto c) {
+          constexpr int e = decltype(c)::value;
+          stage_out(c, s->g[warp][e]);
+        });
+        if (piece1 < stages) continue;  // more pieces of this sub-integration
+      }
+      const int off_s = lane < N ? C::off(lane, N) : 0, off_d = lane < N ? C::off(lane, lane) : 0;
       constexpr int kE = ((8 * NB) * (8 * NB + 1) / 2 + 31) / 32;  // entries per lane
-      const int off_s = lane < N ? C::off(lane, N) : 0;
-      const int off_d = lane < N ? C::off(lane, lane) : 0;
 #pragma unroll 1
-      for (int c0 = 0; c0 < kCW; c0 += kMmEpi) {
+      for (int c0 = 0; c0 < C::kCW; c0 += kMmEpi) {
         const int nu = min(kMmEpi, g.n_chan - (ch0 + c0));  // channels of the group that exist
         if (nu <= 0) break;
         __syncwarp();
-        // registers cannot be indexed: the staging of each group is its own code
+        if constexpr (!C::kLong && NB <= 3) {
 #pragma unroll
-        for (int gr = 0; gr < kCW / kMmEpi; ++gr) {
+        for (int gr = 0; gr < C::kCW / kMmEpi; ++gr) {
           if (gr * kMmEpi != c0) continue;
 #pragma unroll
           for (int u = 0; u < kMmEpi; ++u) {
             const int c = gr * kMmEpi + u;
-            float* sg = s->g[warp][u];
+            float* sg = reinterpret_cast<float*>(s->g[warp][u]);
             auto put = [&](int at, const float* d) {
               *reinterpret_cast<float2*>(sg + at) = make_float2(d[0], d[1]);
             };
@@ -497,29 +621,46 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             }
           }
         }
+        } else if constexpr (!C::kLong) {
+          // registers cannot be indexed: the staging of each group is its own code
+          static_loop<C::kCW / kMmEpi>([&](auto gr) {
+            constexpr int e = decltype(gr)::value * kMmEpi;
+            if (e == c0)
+              static_loop<kMmEpi>([&](auto u) {
+                constexpr int k = decltype(u)::value;
+                stage_out(std::integral_constant<int, e + k>{}, s->g[warp][k]);
+              });
+          });
+        }
+        typename C::Sum(*sg)[C::kG] = s->g[warp] + (C::kLong ? c0 : 0);
         __syncwarp();
-        if (lane < N) {
+        auto beam = [&](int a, int off_s, int off_d) {
 #pragma unroll
           for (int u = 0; u < kMmEpi; ++u) {
-            const int32_t sa = (int)s->g[warp][u][off_s];
-            const int64_t var = (int64_t)n * (int)s->g[warp][u][off_d] - (int64_t)sa * sa;
+            const int32_t sa = (int)sg[u][off_s];
+            const int64_t var = (int64_t)n * (int)sg[u][off_d] - (int64_t)sa * sa;
             float inv = 0.f;
             if (var > 0) {
-              const float vf = i64_to_float(var);
+              const float vf = cov_to_float<C::kLong>(var);
               inv = rsqrtf(vf);
               inv = inv * (1.5f - 0.5f * vf * inv * inv);
             } else if (g.corr && u < nu) {
               atomicAdd(g.degenerate, 1ull);
             }
-            s->row[warp][u][lane] = make_int2(sa, __float_as_int(inv));
+            s->row[warp][u][a] = make_int2(sa, __float_as_int(inv));
           }
+        };
+        if constexpr (NB <= 3) {
+          if (lane < N) beam(lane, off_s, off_d);
+        } else {
+          for (int a = lane; a < N; a += 32) beam(a, C::off(a, N), C::off(a, a));
         }
         __syncwarp();
         const int64_t cell = (int64_t)k * g.n_chan + ch0 + c0;
         if (g.corr) {
           const int np = N * (N + 1) / 2;
           float* dc = g.corr + cell * (int64_t)np + lane;
-#pragma unroll
+#pragma unroll(NB <= 3 ? kE : 2)
           for (int i = 0; i < kE; ++i) {
             if (32 * i >= P) break;
             if (lane + 32 * i < P) {
@@ -530,8 +671,8 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 for (int u = 0; u < kMmEpi; ++u) {
                   const int2 ra = s->row[warp][u][a], rb = s->row[warp][u][b];
                   const int64_t cov =
-                      (int64_t)n * (int)s->g[warp][u][l & 0xffff] - (int64_t)ra.x * rb.x;
-                  const float r = i64_to_float(cov) * __int_as_float(ra.y) * __int_as_float(rb.y);
+                      (int64_t)n * (int)sg[u][l & 0xffff] - (int64_t)ra.x * rb.x;
+                  const float r = cov_to_float<C::kLong>(cov) * __int_as_float(ra.y) * __int_as_float(rb.y);
                   if (u < nu) dc[u * np + 32 * i - a] = a == b ? 1.f : r;
                 }
               }
@@ -548,12 +689,12 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             for (int u = 0; u < kMmEpi; ++u) {
               int64_t v = n;
               if (a < N) {
-                v = (int64_t)(int)s->g[warp][u][l & 0xffff] +
+                v = (int64_t)(int)sg[u][l & 0xffff] +
                     128 * (int64_t)(b == N ? n : s->row[warp][u][a].x + s->row[warp][u][b].x);
                 if (b < N) v += 16384 * n;
               }
               int64_t* o = ds + u * P + 32 * i;
-              if (u < nu) *o = piece0 > 0 ? *o + v : v;
+              if (u < nu) *o = !C::kLong && piece0 > 0 ? *o + v : v;
             }
           }
         }
@@ -628,19 +769,38 @@ bool gram_mma_bulk(const mraid_plan_s* pl, const void* d_data) {
          encode_fn() != nullptr;
 }
 
+// Few beams by plain copies leave long sub-integrations bound by the length
+// of a stage (0.5-0.7 us, whatever its few products), and dp4a with its many
+// small blocks is the faster one: measured at 1000 channels, 2 beams x 3000
+// samples x 12 0.130 ms against 0.183 here, 7 beams x 3000 x 3 0.123 against
+// 0.134-0.166, but 0.231 against 0.192 at 12 sub-integrations (384 items of 32
+// channels), and 0.031 against 0.024 for 4 beams x 64 x 40. Copies of single
+// bytes are slower on dp4a throughout (1001 channels, 2 beams: 0.332 against
+// 0.326; 36 beams x 1000 samples x 20: 5.7 against 1.9).
+bool gram_mma_takes(const mraid_plan_s* pl, const void* d_data) {
+  const mraid_params& p = pl->p;
+  if (!gram_mma_supported(pl)) return false;
+  if (p.n_beam > 7 || p.n_samp_sub < 512 || gram_mma_bulk(pl, d_data)) return true;
+  const bool words =
+      (((uint64_t)p.n_chan | (uint64_t)pl->beam_stride | (uint64_t)(uintptr_t)d_data) & 3) == 0;
+  return !words || (p.n_beam > 2 && (int64_t)p.n_sub * ((p.n_chan + 31) / 32) > pl->sm_count);
+}
+
 bool gram_mma_supported(const mraid_plan_s* pl) {
-  return pl->p.bit_depth == 8 && pl->p.n_beam >= 2 && pl->p.n_beam <= 23;
+  return pl->p.bit_depth == 8 && pl->p.n_beam >= 2 && pl->p.n_beam <= 39;
 }
 
 cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
                             int64_t* d_sums, float* d_corr) {
   const mraid_params& p = pl->p;
-  if (!gram_mma_supported(pl) || (d_corr && p.n_samp_sub > kMmPiece)) return cudaErrorNotSupported;
+  if (!gram_mma_supported(pl) || (d_corr && p.n_samp_sub > kMmLongMax)) return cudaErrorNotSupported;
   MmArgs a;
   a.data = d_data;
   a.beam_stride = pl->beam_stride;
   const uint64_t align = (uint64_t)p.n_chan | (uint64_t)pl->beam_stride | (uint64_t)(uintptr_t)d_data;
   a.vec = align % 8 == 0 ? 8 : (align % 4 == 0 ? 4 : 1);
+  a.data_end = d_data + (int64_t)(p.n_beam - 1) * pl->beam_stride +
+               (int64_t)(sub0 + n_sub) * p.n_samp_sub * p.n_chan;
   a.n_beam = p.n_beam;
   a.n_chan = p.n_chan;
   a.n_samp_sub = p.n_samp_sub;
@@ -657,10 +817,33 @@ cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int s
   // per sample, 64 channels = 100: 128 channels 137 for up to 15 beams, 96
   // channels 113 for 16 to 19; 32 channels, half the warps, 55), the
   // narrower ones leave less of the last round over the SMs empty.
-  const bool narrow = pl->tc_variant & 1;
+  // Sub-integrations of several pieces keep int32 sums of every channel in
+  // shared memory: 64-channel items for 16 beams and more, whose sums leave
+  // the ring of wider ones too shallow.
+  const bool lng = p.n_samp_sub > kMmPiece && p.n_samp_sub <= kMmLongMax;
   const int64_t c64 = item_cost(a, pl->sm_count, 64, 100);
   const int64_t c32 = item_cost(a, pl->sm_count, 32, 55);
-  const int64_t cw = p.n_beam <= 15   ? item_cost(a, pl->sm_count, 128, 137)
+  const int64_t c128 = item_cost(a, pl->sm_count, 128, 137);
+  if (lng) {
+    if (p.n_beam <= 7)
+      return c32 < c128 ? launch_cfg<MmCfg<1, false, 32, 0, 8, true>>(pl, a, tma)
+                        : launch_cfg<MmCfg<1, false, 128, 0, 8, true>>(pl, a, tma);
+    if (p.n_beam <= 15)
+      return c32 < c128 ? launch_cfg<MmCfg<2, false, 32, 0, 8, true>>(pl, a, tma)
+                        : launch_cfg<MmCfg<2, false, 128, 0, 8, true>>(pl, a, tma);
+    if (p.n_beam <= 19)
+      return c32 < c64 ? launch_cfg<MmCfg<3, true, 32, 0, 8, true>>(pl, a, tma)
+                       : launch_cfg<MmCfg<3, true, 64, 0, 8, true>>(pl, a, tma);
+    if (p.n_beam <= 23)
+      return c32 < c64 ? launch_cfg<MmCfg<3, false, 32, 0, 8, true>>(pl, a, tma)
+                       : launch_cfg<MmCfg<3, false, 64, 0, 8, true>>(pl, a, tma);
+    if (p.n_beam <= 31) return launch_cfg<MmCfg<4, false, 32, 0, 4, true>>(pl, a, tma);
+    return launch_cfg<MmCfg<5, false, 32, 0, 4, true>>(pl, a, tma);
+  }
+  if (p.n_beam > 31) return launch_cfg<MmCfg<5, false, 32, 0, 4>>(pl, a, tma);
+  if (p.n_beam > 23) return launch_cfg<MmCfg<4, false, 32, 0, 4>>(pl, a, tma);
+  const bool narrow = pl->tc_variant & 1;
+  const int64_t cw = p.n_beam <= 15   ? c128
                      : p.n_beam <= 19 ? item_cost(a, pl->sm_count, 96, 113)
                                       : INT64_MAX;
   const int pick = narrow ? 64 : (c32 < c64 && c32 < cw ? 32 : (cw <= c64 ? 128 : 64));

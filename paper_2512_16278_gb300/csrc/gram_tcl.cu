@@ -1,14 +1,13 @@
-// gram_tcl.cu - exact augmented Gram sums of 8-bit data for 24..127 beams
+// gram_tcl.cu - exact augmented Gram sums of 8-bit data for 40..127 beams
 // on the tensor cores, channels kept apart by rows.
 //
 // Section 3.2, Eq. 1, for the larger (phased-array-feed) receivers. The
-// channel block-diagonal layout of gram_tc.cu holds at most 23 beams (its
-// accumulators for 16 channels fill TMEM). Here an operand tile holds G
-// channels' beams in 128 rows, R = 128 / G rows each (x - 128 in f16, row
-// N of each channel the row of ones, rows past N zero): G = 4 for up to 31
-// beams, 2 for up to 63, else 1 with R = np = N + 1 rounded up to 16. One
-// MMA (M = 128, K = 16 samples) multiplies the tile by itself (B = its
-// first 128 rows, or np for G = 1); the G diagonal R x R blocks of D are
+// register fragments of gram_mma.cu hold at most 39 beams of four channels
+// per warp. Here an operand tile holds G channels' beams in 128 rows,
+// R = 128 / G rows each (x - 128 in f16, row N of each channel the row of
+// ones, rows past N zero): G = 2 for up to 63 beams, else 1 with R = np =
+// N + 1 rounded up to 16. One MMA (M = 128, K = 16 samples) multiplies the
+// tile by itself (B = its first 128 rows, or np for G = 1); the G diagonal R x R blocks of D are
 // the channels' Gram matrices, the rest is discarded. Fewer, wider MMAs
 // beat one per channel: a tcgen05.mma costs about 90 cycles of issue
 // whatever its N. A CTA keeps nc channels' accumulators in TMEM (512
@@ -16,7 +15,7 @@
 // that run side by side (consecutive work items), the repeated box reads
 // coming from L2.
 //
-// Exactness as in gram_tc.cu: products of centred bytes are integers of
+// Exactness as in gram_mma.cu: products of centred bytes are integers of
 // magnitude <= 2^14 and the FP32 accumulation is exact while a partial sum
 // stays within 2^24, i.e. over at most 1024 samples. Longer
 // sub-integrations are accumulated in TMEM in pieces of <= 1024 samples,
@@ -97,9 +96,8 @@ struct LShape {
   int G, R, gcols;
 };
 __host__ __device__ constexpr LShape l_shape(int n_beam) {
-  return n_beam + 1 <= 32   ? LShape{4, 32, 128}
-         : n_beam + 1 <= 64 ? LShape{2, 64, 128}
-                            : LShape{1, (n_beam + 1 + 15) / 16 * 16, (n_beam + 1 + 15) / 16 * 16};
+  return n_beam + 1 <= 64 ? LShape{2, 64, 128}
+                          : LShape{1, (n_beam + 1 + 15) / 16 * 16, (n_beam + 1 + 15) / 16 * 16};
 }
 __host__ __device__ constexpr uint32_t l_gstride(LShape sh) {
   return (uint32_t)(sh.G * sh.R) * 32u + 16u;
@@ -151,9 +149,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
       : "r"(taddr));
 }
 
-// kAll16: a pass holds all 16 channels of a box (nc = 16), so a converter
-// thread stores both of its channels.
-template <bool kAll16>
 __global__ void __launch_bounds__(kLThreads, 1)
 gram_tcl_kernel(const __grid_constant__ CUtensorMap tmap, LArgs g) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -290,9 +285,9 @@ gram_tcl_kernel(const __grid_constant__ CUtensorMap tmap, LArgs g) {
     // with one ldmatrix .x2 per pair and K step: thread (p, q) = (lane / 4,
     // lane % 4) gets samples 4q..4q+3 of channels p and p + 8 of each beam.
     // Channel c0 + ci of the pass goes to group tile ci / G, rows
-    // R (ci % G) + b, K offset 4q: for nc <= 8 at most one of the thread's
-    // two channels (stored under a predicate), for nc = 16 both. A K step's
-    // loads are issued before its stores.
+    // R (ci % G) + b, K offset 4q: at most one of the thread's two channels,
+    // as nc <= 8 (stored under a predicate). A K step's loads are issued
+    // before its stores.
     const int cw = warp - 2;
     const int p = lane / 4, q = lane % 4;
     const int n_pairs = (N + 1) / 2;
@@ -320,11 +315,9 @@ gram_tcl_kernel(const __grid_constant__ CUtensorMap tmap, LArgs g) {
       const int ncp = l_pass_channels((int)(it % g.passes), nc);
       const int ci0 = p - c0, ci1 = p + 8 - c0;  // channel p / p + 8 in the pass (valid in [0, ncp))
       const bool use0 = ci0 >= 0 && ci0 < ncp, use1 = ci1 >= 0 && ci1 < ncp;
-      // first store: channel p if it is the pass's, else p + 8; second
-      // (nc = 16 only): channel p + 8
+      // channel p if it is the pass's, else p + 8
       const uint32_t ta = chan_off(use0 ? ci0 : (use1 ? ci1 : 0)) + lane_off;
-      const uint32_t tb = chan_off(use1 ? ci1 : 0) + lane_off;
-      const uint32_t pa = (use0 || use1) ? 1u : 0u, pb = (use0 && use1) ? 1u : 0u;
+      const uint32_t pa = (use0 || use1) ? 1u : 0u;
       for (int st = 0; st < stages && ok; ++st, ++cnt) {
         const int us = cnt % kNU, fs = cnt % kLNF;
         ok = mbar_wait(&s->u8_full[us], (cnt / kNU) & 1, g.error, g.wait_ns);
@@ -336,7 +329,6 @@ gram_tcl_kernel(const __grid_constant__ CUtensorMap tmap, LArgs g) {
         for (int ks = 0; ks < kLKs; ++ks) {
           const uint32_t rows = src + (uint32_t)(ks * 16 + (lane & 15)) * 16u;
           const uint32_t kda = dst + (uint32_t)ks * g.ks_stride + ta;
-          const uint32_t kdb = dst + (uint32_t)ks * g.ks_stride + tb;
 #pragma unroll
           for (int j0 = 0; j0 < kLMaxPW; j0 += kLRound) {
             if (cw + kLConvWarps * j0 >= n_pairs) break;
@@ -357,10 +349,6 @@ gram_tcl_kernel(const __grid_constant__ CUtensorMap tmap, LArgs g) {
                 uint32_t lo, hi;
                 u8x4_to_f16(ra, lo, hi);
                 st_shared_v2_if(kda + row, lo, hi, h ? (pa & odd) : pa);
-                if (kAll16) {
-                  u8x4_to_f16(r[jj][2 * h + 1], lo, hi);
-                  st_shared_v2_if(kdb + row, lo, hi, h ? (pb & odd) : pb);
-                }
               }
             }
           }
@@ -474,13 +462,12 @@ gram_tcl_kernel(const __grid_constant__ CUtensorMap tmap, LArgs g) {
 
 // Channels per pass: the most whose accumulators fit TMEM ((nc / G) x gcols
 // <= 512 columns) and whose tables, two f16 stages and an u8 ring of two
-// stages fit shared memory: 16 or 8 for the four- and two-channel tiles
-// (a divisor of 16 that is a multiple of G), any count for one channel per
-// tile (the box's last pass then takes the remaining channels); 0 if none
+// stages fit shared memory: 8 or 4 for the two-channel tiles (a divisor of 16
+// that is a multiple of G), any count for one channel per tile (the box's last pass then takes the remaining channels); 0 if none
 // fits.
 int l_channels(int n_beam, int* n_u8_out) {
   const LShape sh = l_shape(n_beam);
-  for (int nc = 16; nc >= sh.G; nc = sh.G > 1 ? nc / 2 : nc - 1) {
+  for (int nc = 8; nc >= sh.G; nc = sh.G > 1 ? nc / 2 : nc - 1) {
     if ((nc / sh.G) * sh.gcols > (int)kLTmemCols) continue;
     const size_t fixed = 1024 + l_f16_region(l_f16_stage(sh, nc)) + l_acc_bytes(n_beam, nc) +
                          sizeof(SmemL);
@@ -498,7 +485,7 @@ int l_channels(int n_beam, int* n_u8_out) {
 
 bool gram_tcl_supported(const mraid_plan_s* pl, const void* d_data) {
   const mraid_params& p = pl->p;
-  return p.bit_depth == 8 && p.n_beam >= 24 && p.n_beam + 1 <= 128 &&
+  return p.bit_depth == 8 && p.n_beam >= 40 && p.n_beam + 1 <= 128 &&
          p.n_samp_sub % kLT == 0 && p.n_samp_sub <= 65536 && p.n_chan % 16 == 0 &&
          pl->beam_stride % 16 == 0 && (reinterpret_cast<uintptr_t>(d_data) & 15) == 0 &&
          (int64_t)p.n_sub * p.n_samp_sub <= 2147483647ll && l_channels(p.n_beam, nullptr) > 0 &&
@@ -552,17 +539,9 @@ cudaError_t launch_gram_tcl(const mraid_plan_s* pl, const uint8_t* d_data, int s
   const int64_t items = (int64_t)n_sub * (p.n_chan / 16) * a.passes;
   const int grid = (int)(items < pl->sm_count ? items : pl->sm_count);
   cudaError_t e;
-  if (a.nc == 16) {
-    e = cudaFuncSetAttribute(gram_tcl_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e == cudaSuccess && grid > 0)
-      gram_tcl_kernel<true><<<grid, kLThreads, smem, pl->stream>>>(map, a);
-  } else {
-    e = cudaFuncSetAttribute(gram_tcl_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e == cudaSuccess && grid > 0)
-      gram_tcl_kernel<false><<<grid, kLThreads, smem, pl->stream>>>(map, a);
-  }
+  e = cudaFuncSetAttribute(gram_tcl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && grid > 0)
+    gram_tcl_kernel<<<grid, kLThreads, smem, pl->stream>>>(map, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -89,7 +89,7 @@ struct mraid_plan_s {
   cudaEvent_t ev_copied[2] = {nullptr, nullptr};
   cudaEvent_t ev_consumed[2] = {nullptr, nullptr};
   mraid::Profiler prof;
-  bool force_dp4a = false;  // use the CUDA-core Gram even where tcgen05 fits
+  bool force_dp4a = false;  // use the CUDA-core Gram even where the tensor cores fit
   int tc_variant = 0;       // 8-bit Gram up to 23 beams: even = work items by the shape,
                             // odd = always of 64 channels
   unsigned long long wait_ns = 2000000000ull;  // bound of every device wait
@@ -182,18 +182,20 @@ constexpr int kTcVariants = 10;  // 8-bit tensor-core Gram ids (see tc_variant)
 constexpr int kEigVariants = 6;  // register eigensolvers (see eig_variant)
 // float32 samples on the tensor cores (split-bf16 products, gram_tc.cu):
 // correlation only, d_corr relative to sub0
-// Tensor-core Gram for 24..127 beams, one channel per MMA (gram_tcl.cu):
+// Tensor-core Gram for 40..127 beams, one or two channels per MMA (gram_tcl.cu):
 // int64 sums [cell][P] of sub-integrations [sub0, sub0 + n_sub), cells
 // relative to sub0.
 bool gram_tcl_supported(const mraid_plan_s* pl, const void* d_data);
 cudaError_t launch_gram_tcl(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
                             int64_t* d_sums);
-// gram_mma.cu: 8-bit Gram for up to 23 beams, any layout, fused with the
-// correlation (sub-integrations of up to gram_mma_piece samples; longer ones
+// gram_mma.cu: 8-bit Gram for up to 39 beams, any layout, fused with the
+// correlation (sub-integrations of up to kMmPieceMax samples; longer ones
 // give the sums only). gram_mma_bulk: true where the samples come by bulk
 // tensor copies.
-constexpr int kMmPieceMax = 1024;
+constexpr int kMmPieceMax = 127 * 1024;
 bool gram_mma_supported(const mraid_plan_s* pl);
+// supported, and faster than dp4a for the plan's shape and d_data's alignment
+bool gram_mma_takes(const mraid_plan_s* pl, const void* d_data);
 bool gram_mma_bulk(const mraid_plan_s* pl, const void* d_data);
 cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
                             int64_t* d_sums, float* d_corr);

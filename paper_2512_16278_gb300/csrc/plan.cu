@@ -224,9 +224,12 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
     }
     return MRAID_OK;
   }
-  const bool mma = !pl->force_dp4a && gram_mma_supported(pl);
+  const bool mma = !pl->force_dp4a && gram_mma_takes(pl, d_data);
   // profiled by the way the samples come: "gram_tc" for bulk tensor copies
-  const int mma_id = mma && gram_mma_bulk(pl, d_data) ? K_GRAM_TC : K_GRAM;
+  // ("gram_tcl" above 23 beams)
+  const int mma_id = !(mma && gram_mma_bulk(pl, d_data)) ? K_GRAM
+                     : pl->p.n_beam <= 23                ? K_GRAM_TC
+                                                         : K_GRAM_TCL;
   if (mma && pl->p.n_samp_sub <= kMmPieceMax) {
     cudaError_t e = MRAID_PROF(pl, mma_id,
                                launch_gram_mma(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
@@ -784,7 +787,7 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
   for (int v = -1; v < kTcVariants && st == MRAID_OK; ++v) {
     pl->force_dp4a = v < 0;
     pl->tc_variant = v < 0 ? 0 : v;
-    // float32 samples, and 24..127 beams, have one tensor-core kernel each,
+    // float32 samples, and 40..127 beams, have one tensor-core kernel each,
     // timed as variant 0
     if (v >= 0 && (pl->p.bit_depth == 32 ? (v > 0 || !gram_tc_f32_supported(pl, d_data))
                                            : (!gram_mma_supported(pl) &&

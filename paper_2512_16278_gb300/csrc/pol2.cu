@@ -107,7 +107,7 @@ mraid_status pol2_stacked_sums(mraid_plan_s* pl, const void* d_data, int64_t* d_
   v.d_error = pl->d_error;
   v.force_dp4a = pl->force_dp4a;
   cudaError_t e = cudaSuccess;
-  if (!v.force_dp4a && gram_mma_supported(&v)) {
+  if (!v.force_dp4a && gram_mma_takes(&v, d_data)) {
     e = MRAID_PROF(pl, gram_mma_bulk(&v, d_data) ? K_GRAM_TC : K_GRAM,
                    launch_gram_mma(&v, static_cast<const uint8_t*>(d_data), 0, v.p.n_sub,
                                    pl->pol_sums, nullptr));
