@@ -282,11 +282,11 @@ struct alignas(16) ClPart {
   float n, s1, s2, e1;  // n < 2^24: exact; the first moment is s1 + e1
 };
 
-__device__ __forceinline__ void cl_sync() {
-  asm volatile(
-      "barrier.cluster.arrive.release.aligned;\n"
-      "barrier.cluster.wait.acquire.aligned;" ::
-          : "memory");
+__device__ __forceinline__ void cl_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cl_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // A pivot near c: eight significant bits, so that rounding v - pivot depends
 // on v's low bits alone and does not lean one way over cells of like values;
@@ -326,6 +326,9 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
   __shared__ int fit_stop;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = gridDim.x, rank = blockIdx.x;
+  // a CTA's shared memory may be written only once it has started: every CTA
+  // arrives here and waits before its first store to the others
+  if (G > 1) cl_arrive();
   const int64_t base = (int64_t)rank * per;
   const int mine = (int)max((int64_t)0, min((int64_t)per, f.n_cells - base));
   const int nq = (mine + 3) / 4;
@@ -370,7 +373,8 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
   auto cluster3 = [&](int buf, ClPart p) -> ClPart {
     if (G == 1) return p;
     if (warp == 0 && lane < G) cl_store(&part[buf][rank], lane, p);
-    cl_sync();
+    cl_arrive();
+    cl_wait();
     if (warp == 0) {
       p = lane < G ? part[buf][lane] : ClPart{};
 #pragma unroll
@@ -394,6 +398,7 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
   double mu = 0.0, sigma = 0.0, thresh = INFINITY;  // thread 0's
   float used = 0.f, prev = -1.f;
   int fits = 0, converged = 0, pass = 0;
+  if (G > 1) cl_wait();
   for (;; ++pass) {
     // v > thresh for a float v equals v > tf, tf the largest float <= thresh
     const float tf = __double2float_rd(thresh);
