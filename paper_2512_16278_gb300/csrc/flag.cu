@@ -265,11 +265,18 @@ __global__ void __launch_bounds__(kFlagThreads) flag_kernel(FlagArgs f) {
 // 868 352 cells (16 CTAs) the cooperative kernel, 102 us.
 //
 // Sums are taken about a pivot (the last fit's mean; for the first fit the
-// mean of the block's first cells), so the variance does not cancel and FP32
-// suffices up to the cluster's total: a fixed tree over lanes, warps and
-// CTAs, the same bits in every CTA. The first moment carries its rounding
-// errors beside it (two floats; the mean is good to 1e-9, and FP64 sums would
-// cost more than the rest of a pass). The fit itself is FP64.
+// mean of the block's first cells): four cells in FP32, then two floats per
+// moment (value and rounding error) through a fixed tree over lanes, warps and
+// CTAs, the same bits in every CTA. FP64 sums would cost more than the rest of
+// a pass; the fit itself is FP64. The cells' own roundings leave the variance
+// s2 / n - m^2 (m the mean's distance from the pivot) an error of 1e-7 s2 / n at
+// most, so it is only used where it is at least a tenth of s2 / n. Where it is
+// less (the last threshold took out cells that had moved the mean by more than
+// three deviations, or the first cells were unlike the rest) the sums are taken
+// again about the new mean, at the same threshold.
+// Against one FP32 sum for s2 the second float and its tree cost 10 us of 75 at
+// 819 200 cells and nothing at 1 024 (two-sums of eight cells instead of four
+// gained 1 us).
 //
 // A cell out of the fit is marked in the shared copy by a NaN of its own
 // (kMasked, kOutside); NaNs of the caller's are made the canonical one.
@@ -278,8 +285,10 @@ constexpr int kClCells = 53 * 1024;  // per CTA: 212 KB of shared memory
 constexpr int kClMaxCtas = 16;
 constexpr int kMasked = 0x7ffffffe, kOutside = 0x7fffffff;  // as int bits: above every other cell
 
+constexpr int kClMoves = 8;  // pivots per fit: each lies 1e7 times closer to the mean
+
 struct alignas(16) ClPart {
-  float n, s1, s2, e1;  // n < 2^24: exact; the first moment is s1 + e1
+  float n, s1, s2, e1, e2;  // n < 2^24: exact; the moments are s1 + e1 and s2 + e2
 };
 
 __device__ __forceinline__ void cl_arrive() {
@@ -288,11 +297,13 @@ __device__ __forceinline__ void cl_arrive() {
 __device__ __forceinline__ void cl_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// A pivot near c: eight significant bits, so that rounding v - pivot depends
-// on v's low bits alone and does not lean one way over cells of like values;
-// no shift for infinities and NaN.
+// A pivot near c: sixteen significant bits, so that v - pivot is exact for v
+// from pivot / 2 to 256 pivot (to 2 pivot by Sterbenz's lemma, beyond as a
+// multiple of v's last bit) and, for smaller v, rounds by v's low bits alone:
+// it does not lean one way over cells of like values. No shift for
+// infinities and NaN.
 __device__ __forceinline__ float pivot_near(float c) {
-  return fabsf(c) < 1e30f ? __uint_as_float(__float_as_uint(c) & 0xffff0000u) : 0.f;
+  return fabsf(c) < 1e30f ? __uint_as_float(__float_as_uint(c) & 0xffffff00u) : 0.f;
 }
 // s + e = a + b exactly (Knuth's two-sum)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -302,11 +313,17 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 }
 // one level of a butterfly over the lanes
 __device__ __forceinline__ void add_lanes(ClPart& p, int o) {
-  const float n = __shfl_xor_sync(0xffffffffu, p.n, o), s2 = __shfl_xor_sync(0xffffffffu, p.s2, o);
+  const float n = __shfl_xor_sync(0xffffffffu, p.n, o);
   const float s1 = __shfl_xor_sync(0xffffffffu, p.s1, o), e1 = __shfl_xor_sync(0xffffffffu, p.e1, o);
-  float s, e;
-  two_sum(p.s1, s1, s, e);
-  p = ClPart{p.n + n, s, p.s2 + s2, e + (p.e1 + e1)};
+  const float s2 = __shfl_xor_sync(0xffffffffu, p.s2, o), e2 = __shfl_xor_sync(0xffffffffu, p.e2, o);
+  float t1, r1, t2, r2;
+  two_sum(p.s1, s1, t1, r1);
+  two_sum(p.s2, s2, t2, r2);
+  p = ClPart{p.n + n, t1, t2, r1 + (p.e1 + e1), r2 + (p.e2 + e2)};
+}
+// s + e (no error term beside an infinity or NaN)
+__device__ __forceinline__ double moment(float s, float e) {
+  return (double)s + (isfinite(s) ? (double)e : 0.0);
 }
 // part (in this CTA's shared memory) of CTA `rank`
 __device__ __forceinline__ void cl_store(ClPart* part, int rank, const ClPart& p) {
@@ -315,6 +332,7 @@ __device__ __forceinline__ void cl_store(ClPart* part, int rank, const ClPart& p
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(r), "f"(p.n), "f"(p.s1),
                "f"(p.s2), "f"(p.e1)
                : "memory");
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r + 16), "f"(p.e2) : "memory");
 }
 
 __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f, int per, int vec) {
@@ -387,7 +405,7 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
   {
     const bool use = tid < f.n_cells && !(f.keep && f.keep[tid % f.n_chan]);
     const float v = use ? f.stat[tid] : 0.f;
-    const ClPart p = block3(ClPart{use ? 1.f : 0.f, v, 0.f, 0.f});
+    const ClPart p = block3(ClPart{use ? 1.f : 0.f, v});
     if (tid == 0) {
       const float c = p.s1 / fmaxf(p.n, 1.f);
       fit_pivot = pivot_near(c);
@@ -397,18 +415,18 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
   float pivot = fit_pivot;
   double mu = 0.0, sigma = 0.0, thresh = INFINITY;  // thread 0's
   float used = 0.f, prev = -1.f;
-  int fits = 0, converged = 0, pass = 0;
+  int fits = 0, converged = 0, pass = 0, moves = 0;
   if (G > 1) cl_wait();
   for (;; ++pass) {
     // v > thresh for a float v equals v > tf, tf the largest float <= thresh
     const float tf = __double2float_rd(thresh);
     int cnt = 0;
-    float s1 = 0.f, s2 = 0.f, e1 = 0.f;
+    float s1 = 0.f, s2 = 0.f, e1 = 0.f, e2 = 0.f;
 #pragma unroll 4
     for (int q = tid; q < nq; q += kClThreads) {
       int4 w = quads[q];
       bool changed = false;
-      float quad = 0.f;
+      float quad = 0.f, quad2 = 0.f;
       auto cell = [&](int& x) {
         const float v = __int_as_float(x);
         if (v > tf) {  // false for the marks
@@ -418,7 +436,7 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
           const float d = v - pivot;
           ++cnt;
           quad += d;
-          s2 = fmaf(d, d, s2);
+          quad2 = fmaf(d, d, quad2);
         }
       };
       cell(w.x);
@@ -429,10 +447,13 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
       float e;
       two_sum(s1, quad, s1, e);
       e1 += e;
+      two_sum(s2, quad2, s2, e);
+      e2 += e;
     }
-    const ClPart p = cluster3(pass & 1, block3(ClPart{(float)cnt, s1, s2, e1}));
+    const ClPart p = cluster3(pass & 1, block3(ClPart{(float)cnt, s1, s2, e1, e2}));
     if (tid == 0) {
       int stop = 0;
+      bool again = false;
       if (pass >= 1 && p.n == prev) {  // the last threshold masked nothing
         converged = 1;
         stop = 1;
@@ -446,16 +467,29 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
         converged = 1;
         stop = 1;
       } else {
-        const double inv = 1.0 / (double)p.n, m = ((double)p.s1 + (isfinite(p.s1) ? (double)p.e1 : 0.0)) * inv;
+        const double inv = 1.0 / (double)p.n;
+        const double m = moment(p.s1, p.e1) * inv, q = moment(p.s2, p.e2) * inv;
         mu = (double)pivot + m;
-        sigma = sqrt(fmax((double)p.s2 * inv - m * m, 0.0));
-        thresh = mu + f.k_sigma * sigma;
-        used = prev = p.n;
-        ++fits;
+        fit_pivot = pivot_near((float)mu);
+        if (m * m > 0.9 * q && moves < kClMoves) {
+          // too far: the same cells about the new mean, by all its bits where
+          // the coarse pivot is the one that was too far
+          if (moves > 0 || fit_pivot == pivot) fit_pivot = (float)mu;
+          again = fit_pivot != pivot;
+        }
+        if (again) {
+          ++moves;
+        } else {
+          sigma = sqrt(fmax(q - m * m, 0.0));
+          thresh = mu + f.k_sigma * sigma;
+          used = prev = p.n;
+          moves = 0;
+          fit_pivot = pivot_near((float)mu);
+          ++fits;
+        }
       }
       fit_thresh = thresh;
       fit_stop = stop;
-      fit_pivot = pivot_near((float)mu);
     }
     __syncthreads();
     thresh = fit_thresh;
@@ -492,7 +526,7 @@ __global__ void __launch_bounds__(kClThreads, 1) flag_cluster_kernel(FlagArgs f,
     }
   }
   // the buffer of the pass before: a CTA may still read the last pass's
-  const ClPart p = cluster3((pass + 1) & 1, block3(ClPart{(float)hits, (float)near, 0.f, 0.f}));
+  const ClPart p = cluster3((pass + 1) & 1, block3(ClPart{(float)hits, (float)near}));
   if (rank == 0 && tid == 0) {
     mraid_flag_info* o = f.info;
     o->mu = mu;
