@@ -810,7 +810,11 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
     pl->force_dp4a = save_dp4a;
     pl->tc_variant = save_v;
   }
-  // Jacobi stage on the correlations just computed
+  // Eigensolver stage on the correlations just computed, with eigenvalues:
+  // without them variants 4 and 5 leave out the kernel in which they differ.
+  // They go to the sums' buffer, which the Gram stage is done with (P int64 a
+  // cell, more than N floats).
+  float* evals = reinterpret_cast<float*>(pl->ws.sums);
   int best_e = pl->eig_variant;
   if (st == MRAID_OK) {
     best = 1e30f;
@@ -819,7 +823,7 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
       float ms = 0.f;
       st = time_runs(pl, reps, e0, e1,
                      [&]() -> mraid_status {
-                       cudaError_t le = launch_eig(pl, pl->ws.corr, pl->n_cells, nullptr, nullptr, stat);
+                       cudaError_t le = launch_eig(pl, pl->ws.corr, pl->n_cells, evals, nullptr, stat);
                        return le == cudaSuccess ? MRAID_OK : cuda_fail(le, "eig launch");
                      },
                      &ms);
