@@ -285,23 +285,25 @@ mraid_status mraid_run_bandpass(mraid_plan_t plan, const void* d_data,
 
 /* Autotuner (the paper has no counterpart; it picks among this library's
  * kernel variants). Times, `reps` runs each on d_data, every Gram variant
- * that fits the plan's shape (for 8-bit samples and up to 39 beams ten ids:
- * even ones choose the channels per work item by the shape, odd ones take 64
- * for up to 23 beams; and the CUDA-core Gram) and the register
+ * that fits the plan's shape (the CUDA-core Gram, the tensor-core Gram and,
+ * for 8-bit samples and up to 23 beams, its form of 64 channels per work item
+ * where the shape's own choice is another) and the register
  * eigensolvers (Jacobi rounds in a loop; the Jacobi sweep unrolled;
  * Householder tridiagonalisation + implicit QR in two code layouts), and
  * keeps the fastest of each for this plan. *gram_choice: -1 = CUDA-core,
- * 0..9 tensor-core variants; *eig_choice: 0..5. report (may be NULL) receives "g<id>:ms;e<id>:ms;...".
+ * 0 and 1 tensor-core variants; *eig_choice: 0..5 (timed with eigenvalues).
+ * report (may be NULL) receives "g<id>:ms;e<id>:ms;...", for 8-bit samples and
+ * up to 39 beams with the ids 1..9 that are aliases (see mraid_set_variant).
  * Synchronous. */
 mraid_status mraid_autotune(mraid_plan_t plan, const void* d_data, int32_t reps,
                             int32_t* gram_choice, int32_t* eig_choice, char* report,
                             int32_t report_len);
 
 /* Select variants by id (e.g. from a tuning cache). Gram: -1 = CUDA-core,
- * 0..9 tensor-core Gram: for up to 23 beams even ids choose the channels per
- * work item by the shape and odd ids take 64; for 24..127 beams any id >= 0
- * selects the tensor-core Gram of that beam count (exact in pieces of <= 1024
- * samples).
+ * 0 = the tensor-core Gram; 1 = the same with 64 channels per work item, for
+ * 8-bit samples, up to 23 beams and sub-integrations of at most 1024 or more
+ * than 127 x 1024 samples (elsewhere an alias of 0); 2..9 = aliases of 0, kept
+ * for programs that name the kernels of earlier versions.
  * Eigensolver (beam counts with a one-thread-per-matrix kernel: 2, 3, 4, 13,
  * 19; other counts always use the warp-per-matrix Jacobi): 0 = Jacobi,
  * looped rounds; 1 = Jacobi, unrolled sweep; 2 = Householder reduction to

@@ -470,12 +470,17 @@ def tune_key(n_beam: int, n_chan: int, n_samp_sub: int, bit_depth: int = 8) -> s
     return f"{n_beam},{n_chan},{n_samp_sub},{'u8' if bit_depth == 8 else 'f32'}"
 
 
+# Version of the kernels that the ids in a tuning cache stand for; a record of
+# another version is measured again.
+TUNE_VERSION = 2
+
+
 def tune(plan: int, d_data, n_beam: int, n_chan: int, n_samp_sub: int,
          cache_path: Optional[str] = None, reps: int = 3, bit_depth: int = 8):
     """Pick the Gram and eigensolver variants for this shape: from the JSON
     tuning cache (keyed by beams, channels, samples per sub-integration and
-    sample type, which must be the plan's bit_depth) if it holds the shape,
-    else by mraid_autotune, recording the result.
+    sample type, which must be the plan's bit_depth) if it holds the shape for
+    these kernels (TUNE_VERSION), else by mraid_autotune, recording the result.
     Returns (gram variant, eigensolver variant)."""
     import json
     key = tune_key(n_beam, n_chan, n_samp_sub, bit_depth)
@@ -483,14 +488,14 @@ def tune(plan: int, d_data, n_beam: int, n_chan: int, n_samp_sub: int,
     if cache_path and os.path.exists(cache_path):
         with open(cache_path) as f:
             cache = json.load(f)
-    if key in cache:
+    if key in cache and cache[key].get("version") == TUNE_VERSION:
         g, e = int(cache[key]["gram"]), int(cache[key]["jacobi"])
         mraid_set_variant(plan, g)
         mraid_set_eig_variant(plan, e)
         return g, e
     (g, e), times = mraid_autotune(plan, d_data, reps)
     if cache_path:
-        cache[key] = {"gram": g, "jacobi": e, "ms": times}
+        cache[key] = {"gram": g, "jacobi": e, "ms": times, "version": TUNE_VERSION}
         tmp = cache_path + f".{os.getpid()}.tmp"
         with open(tmp, "w") as f:
             json.dump(cache, f, indent=1, sort_keys=True)

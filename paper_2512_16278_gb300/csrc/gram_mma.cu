@@ -752,9 +752,31 @@ cudaError_t launch_cfg(const mraid_plan_s* pl, MmArgs& a, bool tma) {
 // Time of a launch with work items of `width` channels, in arbitrary units:
 // rounds of items over the SMs, each as long as its width over the rate of
 // that width (percent of the 64-channel one).
-int64_t item_cost(const MmArgs& a, int sm_count, int width, int rate) {
-  const int64_t items = (int64_t)a.n_sub * ((a.n_chan + width - 1) / width);
+int64_t item_cost(int n_sub, int n_chan, int sm_count, int width, int rate) {
+  const int64_t items = (int64_t)n_sub * ((n_chan + width - 1) / width);
   return (items + sm_count - 1) / sm_count * width * 1000 / rate;
+}
+
+// Channels of a work item: the wider ones run more warps per SM (measured
+// per sample, 64 channels = 100: 128 channels 137 for up to 15 beams, 96
+// channels 113 for 16 to 19; 32 channels, half the warps, 55), the narrower
+// ones leave less of the last round over the SMs empty. Sub-integrations of
+// several pieces keep int32 sums of every channel in shared memory:
+// 64-channel items for 16 beams and more, whose sums leave the ring of wider
+// ones too shallow. From 24 beams on 32.
+int item_width(const mraid_plan_s* pl, int n_sub) {
+  const mraid_params& p = pl->p;
+  if (p.n_beam > 23) return 32;
+  auto cost = [&](int width, int rate) {
+    return item_cost(n_sub, p.n_chan, pl->sm_count, width, rate);
+  };
+  const int64_t c32 = cost(32, 55), c64 = cost(64, 100);
+  const bool lng = p.n_samp_sub > kMmPiece && p.n_samp_sub <= kMmLongMax;
+  if (lng && p.n_beam <= 15) return c32 < cost(128, 137) ? 32 : 128;
+  if (lng || p.n_beam > 19) return c32 < c64 ? 32 : 64;
+  const int wide = p.n_beam <= 15 ? 128 : 96;
+  const int64_t cw = p.n_beam <= 15 ? cost(128, 137) : cost(96, 113);
+  return c32 < c64 && c32 < cw ? 32 : (cw <= c64 ? wide : 64);
 }
 
 }  // namespace
@@ -786,6 +808,12 @@ bool gram_mma_takes(const mraid_plan_s* pl, const void* d_data) {
   return !words || (p.n_beam > 2 && (int64_t)p.n_sub * ((p.n_chan + 31) / 32) > pl->sm_count);
 }
 
+bool gram_mma_has_forms(const mraid_plan_s* pl) {
+  const mraid_params& p = pl->p;
+  return p.n_beam <= 23 && (p.n_samp_sub <= kMmPiece || p.n_samp_sub > kMmLongMax) &&
+         item_width(pl, p.n_sub) != 64;
+}
+
 bool gram_mma_supported(const mraid_plan_s* pl) {
   return pl->p.bit_depth == 8 && pl->p.n_beam >= 2 && pl->p.n_beam <= 39;
 }
@@ -813,40 +841,26 @@ cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int s
   a.wait_ns = pl->wait_ns;
   a.withhold = pl->inject_withhold;
   const bool tma = gram_mma_bulk(pl, d_data);
-  // The width of a work item: the wider ones run more warps per SM (measured
-  // per sample, 64 channels = 100: 128 channels 137 for up to 15 beams, 96
-  // channels 113 for 16 to 19; 32 channels, half the warps, 55), the
-  // narrower ones leave less of the last round over the SMs empty.
-  // Sub-integrations of several pieces keep int32 sums of every channel in
-  // shared memory: 64-channel items for 16 beams and more, whose sums leave
-  // the ring of wider ones too shallow.
   const bool lng = p.n_samp_sub > kMmPiece && p.n_samp_sub <= kMmLongMax;
-  const int64_t c64 = item_cost(a, pl->sm_count, 64, 100);
-  const int64_t c32 = item_cost(a, pl->sm_count, 32, 55);
-  const int64_t c128 = item_cost(a, pl->sm_count, 128, 137);
+  const int pick = pl->tc_variant == 1 && !lng ? 64 : item_width(pl, n_sub);
   if (lng) {
     if (p.n_beam <= 7)
-      return c32 < c128 ? launch_cfg<MmCfg<1, false, 32, 0, 8, true>>(pl, a, tma)
+      return pick == 32 ? launch_cfg<MmCfg<1, false, 32, 0, 8, true>>(pl, a, tma)
                         : launch_cfg<MmCfg<1, false, 128, 0, 8, true>>(pl, a, tma);
     if (p.n_beam <= 15)
-      return c32 < c128 ? launch_cfg<MmCfg<2, false, 32, 0, 8, true>>(pl, a, tma)
+      return pick == 32 ? launch_cfg<MmCfg<2, false, 32, 0, 8, true>>(pl, a, tma)
                         : launch_cfg<MmCfg<2, false, 128, 0, 8, true>>(pl, a, tma);
     if (p.n_beam <= 19)
-      return c32 < c64 ? launch_cfg<MmCfg<3, true, 32, 0, 8, true>>(pl, a, tma)
-                       : launch_cfg<MmCfg<3, true, 64, 0, 8, true>>(pl, a, tma);
+      return pick == 32 ? launch_cfg<MmCfg<3, true, 32, 0, 8, true>>(pl, a, tma)
+                        : launch_cfg<MmCfg<3, true, 64, 0, 8, true>>(pl, a, tma);
     if (p.n_beam <= 23)
-      return c32 < c64 ? launch_cfg<MmCfg<3, false, 32, 0, 8, true>>(pl, a, tma)
-                       : launch_cfg<MmCfg<3, false, 64, 0, 8, true>>(pl, a, tma);
+      return pick == 32 ? launch_cfg<MmCfg<3, false, 32, 0, 8, true>>(pl, a, tma)
+                        : launch_cfg<MmCfg<3, false, 64, 0, 8, true>>(pl, a, tma);
     if (p.n_beam <= 31) return launch_cfg<MmCfg<4, false, 32, 0, 4, true>>(pl, a, tma);
     return launch_cfg<MmCfg<5, false, 32, 0, 4, true>>(pl, a, tma);
   }
   if (p.n_beam > 31) return launch_cfg<MmCfg<5, false, 32, 0, 4>>(pl, a, tma);
   if (p.n_beam > 23) return launch_cfg<MmCfg<4, false, 32, 0, 4>>(pl, a, tma);
-  const bool narrow = pl->tc_variant & 1;
-  const int64_t cw = p.n_beam <= 15   ? c128
-                     : p.n_beam <= 19 ? item_cost(a, pl->sm_count, 96, 113)
-                                      : INT64_MAX;
-  const int pick = narrow ? 64 : (c32 < c64 && c32 < cw ? 32 : (cw <= c64 ? 128 : 64));
   if (p.n_beam <= 7)
     return pick == 32   ? launch_cfg<MmCfg<1, false, 32, 0>>(pl, a, tma)
            : pick == 64 ? launch_cfg<MmCfg<1, false, 64, 0>>(pl, a, tma)

@@ -90,8 +90,8 @@ struct mraid_plan_s {
   cudaEvent_t ev_consumed[2] = {nullptr, nullptr};
   mraid::Profiler prof;
   bool force_dp4a = false;  // use the CUDA-core Gram even where the tensor cores fit
-  int tc_variant = 0;       // 8-bit Gram up to 23 beams: even = work items by the shape,
-                            // odd = always of 64 channels
+  int tc_variant = 0;       // 8-bit Gram up to 23 beams: 1 = work items of 64 channels, any
+                            // other id = by the shape
   unsigned long long wait_ns = 2000000000ull;  // bound of every device wait
   long long inject_withhold = -1;  // MRAID_FAULT_WITHHOLD_STAGE: stage to skip, or -1
   bool inject_alloc = false;       // MRAID_FAULT_ALLOC armed
@@ -178,7 +178,7 @@ cudaError_t launch_gram_f32(const mraid_plan_s* pl, const float* d_data, int sub
 bool gram_tc_pol2_supported(const mraid_plan_s* pl, const void* d_data);
 cudaError_t launch_gram_tc_pol2(const mraid_plan_s* pl, const uint8_t* d_data, int64_t* d_sums,
                                 float* d_corr);
-constexpr int kTcVariants = 10;  // 8-bit tensor-core Gram ids (see tc_variant)
+constexpr int kTcVariants = 10;  // 8-bit tensor-core Gram ids: 0, 1 and aliases of 0
 constexpr int kEigVariants = 6;  // register eigensolvers (see eig_variant)
 // float32 samples on the tensor cores (split-bf16 products, gram_tc.cu):
 // correlation only, d_corr relative to sub0
@@ -194,6 +194,8 @@ cudaError_t launch_gram_tcl(const mraid_plan_s* pl, const uint8_t* d_data, int s
 // tensor copies.
 constexpr int kMmPieceMax = 127 * 1024;
 bool gram_mma_supported(const mraid_plan_s* pl);
+// true where variants 0 and 1 are different launches
+bool gram_mma_has_forms(const mraid_plan_s* pl);
 // supported, and faster than dp4a for the plan's shape and d_data's alignment
 bool gram_mma_takes(const mraid_plan_s* pl, const void* d_data);
 bool gram_mma_bulk(const mraid_plan_s* pl, const void* d_data);

@@ -784,24 +784,30 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
   const int save_v = pl->tc_variant;
   float best = 1e30f;
   int best_g = -2;
-  for (int v = -1; v < kTcVariants && st == MRAID_OK; ++v) {
+  // Each launch is timed once: id 1 only where it differs from 0, and id 0
+  // not where the rule takes the CUDA cores anyway. The report has the ids
+  // that are aliases too.
+  const bool mma = gram_mma_supported(pl);
+  const bool tc = pl->p.bit_depth == 32 ? gram_tc_f32_supported(pl, d_data)
+                  : mma                 ? gram_mma_takes(pl, d_data)
+                                        : gram_tcl_supported(pl, d_data);
+  const int last = tc ? (mma && gram_mma_has_forms(pl) ? 1 : 0) : -1;
+  float ms[3] = {};  // of ids -1, 0, 1
+  for (int v = -1; v <= last && st == MRAID_OK; ++v) {
     pl->force_dp4a = v < 0;
     pl->tc_variant = v < 0 ? 0 : v;
-    // float32 samples, and 40..127 beams, have one tensor-core kernel each,
-    // timed as variant 0
-    if (v >= 0 && (pl->p.bit_depth == 32 ? (v > 0 || !gram_tc_f32_supported(pl, d_data))
-                                           : (!gram_mma_supported(pl) &&
-                                              (v > 0 || !gram_tcl_supported(pl, d_data)))))
-      continue;
-    float ms = 0.f;
     st = time_runs(pl, reps, e0, e1,
-                   [&] { return ccm_range(pl, d_data, 0, pl->p.n_sub, nullptr, pl->ws.corr); }, &ms);
-    if (st != MRAID_OK) break;
-    note('g', v, ms);
-    if (ms < best) {
-      best = ms;
+                   [&] { return ccm_range(pl, d_data, 0, pl->p.n_sub, nullptr, pl->ws.corr); },
+                   &ms[v + 1]);
+    if (st == MRAID_OK && ms[v + 1] < best) {
+      best = ms[v + 1];
       best_g = v;
     }
+  }
+  if (st == MRAID_OK) {
+    if (mma && !tc) best_g = 0;  // the rule: other buffers of the plan may suit the tensor cores
+    for (int v = -1; v < (mma ? kTcVariants : last + 1); ++v)
+      note('g', v, ms[v < 0 || !tc ? 0 : (v == 1 && last == 1 ? 2 : 1)]);
   }
   if (st == MRAID_OK && best_g >= -1) {
     pl->force_dp4a = best_g < 0;
