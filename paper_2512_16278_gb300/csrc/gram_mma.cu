@@ -34,8 +34,8 @@
 // at 4.7-4.8 TB/s on GB300, 64-byte ones at 6.3-6.7, 128-byte ones at 7.1.
 // Layouts that no tensor map takes (odd channel counts, misaligned buffers)
 // fill the same ring by cp.async, or at odd addresses from pairs of aligned
-// words (byte by byte, 36 beams x 1001 channels x 1000 samples x 20 took 4.4
-// ms, so 1.96).
+// words (36 beams x 1001 channels x 1000 samples x 20 1.15 ms, on dp4a 5.7; x
+// 1000 channels, in 8-byte copies, 0.64).
 //
 // Measured on GB300 (50 sub-integrations x 4096 channels x 1024 samples):
 // 19 beams 0.89 ms (4.5 TB/s of samples; the tcgen05 kernel 1.20 ms), 13
@@ -263,9 +263,16 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       tma_load_3d(dst + box_a, &map_b, ch0 + C::kChA, t0, 0, &s->full[slot]);
   };
   // the same by every thread's own copies, for layouts that no tensor map
-  // takes; a thread fills one place of every beam (or of every other one),
-  // worked out anew each time: kept in registers it made few beams 15 %
-  // faster but 19 beams x 1000 x 1000 x 40 0.52 ms instead of 0.38 (spills)
+  // takes; a stage has kPlaces8 or kPlaces4 places of 8 or 4 bytes a beam, and
+  // the kGroups8 or kGroups4 groups of that many threads share the beams. A
+  // thread's place is worked out anew each time: kept in registers it made few
+  // beams 15 % faster but 19 beams x 1000 x 1000 x 40 0.52 ms instead of 0.38
+  // (spills)
+  constexpr int kPlaces8 = C::kCh / 8 * kMmT, kPlaces4 = C::kCh / 4 * kMmT;
+  constexpr int kGroups8 = C::kThreads / kPlaces8, kGroups4 = C::kThreads / kPlaces4;
+  static_assert(kGroups8 * kPlaces8 == C::kThreads && kGroups4 * kPlaces4 == C::kThreads,
+                "every thread has a place, and no two the same");
+  const int group4 = kGroups4 > 1 ? threadIdx.x / kPlaces4 : 0;
   int f_it = blockIdx.x, f_st = 0, f_slot = 0;  // next stage to fill
   auto fill = [&](int r) {
     const int v = g.vec, words = v == 8 ? C::kCh / 8 : C::kCh / 4;
@@ -279,10 +286,10 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                    row * pitch + ((c16 ^ swizzle(pitch, row)) << 4) + (cc & 15);
     const bool mine = row < nv && ch < g.n_chan && !(blockIdx.x == 0 && r == g.withhold);
     if (v == 8) {
-      for (int b = threadIdx.x / (words * kMmT); b < N; b += 2)
+      for (int b = threadIdx.x / kPlaces8; b < N; b += kGroups8)
         if (mine) copy_async<8>(dst + b * kMmT * pitch, src + b * g.beam_stride);
     } else if (v == 4) {
-      for (int b = 0; b < N; ++b)
+      for (int b = group4; b < N; b += kGroups4)
         if (mine) copy_async<4>(dst + b * kMmT * pitch, src + b * g.beam_stride);
     } else if (mine) {
       const int nc = g.n_chan - ch;
@@ -292,7 +299,7 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       auto word = [](const uint8_t* p) { return p - (reinterpret_cast<uintptr_t>(p) & 3); };
       if (nc >= 4 && word(src) >= g.data &&
           word(src + (N - 1) * g.beam_stride) + 8 <= g.data_end) {
-        for (int b0 = 0; b0 < N; b0 += 8) {
+        for (int b0 = 8 * group4; b0 < N; b0 += 8 * kGroups4) {
           uint32_t lo[8], hi[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -311,7 +318,7 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
       } else {
 #pragma unroll 4
-        for (int b = 0; b < N; ++b) {
+        for (int b = group4; b < N; b += kGroups4) {
           const uint8_t* p = src + b * g.beam_stride;
           uint32_t x = p[0];
           if (nc > 1) x |= (uint32_t)p[1] << 8;
@@ -798,7 +805,7 @@ bool gram_mma_bulk(const mraid_plan_s* pl, const void* d_data) {
 // 0.134-0.166, but 0.231 against 0.192 at 12 sub-integrations (384 items of 32
 // channels), and 0.031 against 0.024 for 4 beams x 64 x 40. Copies of single
 // bytes are slower on dp4a throughout (1001 channels, 2 beams: 0.332 against
-// 0.326; 36 beams x 1000 samples x 20: 5.7 against 1.9).
+// 0.326; 36 beams x 1000 samples x 20: 5.7 against 1.15).
 bool gram_mma_takes(const mraid_plan_s* pl, const void* d_data) {
   const mraid_params& p = pl->p;
   if (!gram_mma_supported(pl)) return false;
