@@ -342,7 +342,7 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   if constexpr (kTma) {
     if (threadIdx.x == 0) {
       for (int i = 0; i < D && i < total; ++i) issue(i);
-      last_issued = D - 1;
+      last_issued = min(D, total) - 1;
     }
   } else {
     for (int i = 0; i < D && i < total; ++i) fill(i);
