@@ -272,6 +272,15 @@ __global__ void corr_from_sums_kernel(const int64_t* __restrict__ sums, int64_t 
 
 }  // namespace
 
+void gram_u8_shape(int n_beam, int n_chan, int* cpb_out, int* tiles) {
+  const int T1 = (n_beam + 1 + 3) / 4;
+  *tiles = T1 * (T1 + 1) / 2;
+  // channels per block: as many as fit 4 tasks per thread, multiple of 4
+  int cpb = (4 * kGramThreads) / *tiles;
+  cpb = cpb >= 32 ? 32 : (cpb >= 4 ? (cpb / 4) * 4 : (cpb < 1 ? 1 : cpb));
+  *cpb_out = cpb > n_chan ? n_chan : cpb;
+}
+
 cudaError_t launch_gram_u8(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
                            int64_t* d_sums) {
   GramArgs g;
@@ -282,12 +291,8 @@ cudaError_t launch_gram_u8(const mraid_plan_s* pl, const uint8_t* d_data, int su
   g.n_samp_sub = pl->p.n_samp_sub;
   g.sub0 = sub0;
   g.R = ((g.n_beam + 1 + 3) / 4) * 4;
-  const int T1 = g.R / 4;
-  g.tiles = T1 * (T1 + 1) / 2;
-  // channels per block: as many as fit 4 tasks per thread, multiple of 4
-  int cpb = (4 * kGramThreads) / g.tiles;
-  cpb = cpb >= 32 ? 32 : (cpb >= 4 ? (cpb / 4) * 4 : (cpb < 1 ? 1 : cpb));
-  if (cpb > g.n_chan) cpb = g.n_chan;
+  int cpb;
+  gram_u8_shape(g.n_beam, g.n_chan, &cpb, &g.tiles);
   g.cpb = cpb;
   g.ntask = cpb * g.tiles;
   g.cs = g.R * kRS + 1;

@@ -85,6 +85,11 @@ struct MmCfg {
   static constexpr int NB = NB_, kChA = A_, kChB = B_, kCh = A_ + B_;
   static constexpr bool kHalf = kHalf_;
   static constexpr int kWarps = kCh / kCW, kThreads = 32 * kWarps;
+  // CTAs per SM where there are more items than SMs: four warps leave an SM
+  // idle between the steps of their chain (with one CTA, 19 beams x 16 channels
+  // x 1024 samples x 250 took 81 us, so 55; 7 beams x 24 channels x 166 95 and
+  // 54)
+  static constexpr int kCtas = (kWarps > 4 ? 1 : (NB_ == 1 ? 3 : 2)) * (kWarps == 2 ? 2 : 1);
   static constexpr int kTile = kMmT * kCh;  // bytes of one beam in a stage
   // One channel's products in the epilogue, in floats: per block row pair
   // (2p, 2p + 1) the 8 x 8 of the diagonal block 2p, then 16 x 8 for every
@@ -115,8 +120,9 @@ struct MmCfg {
   }
   static constexpr size_t kFixed = 1024 + sizeof(Shared);
   static constexpr int stage_bytes(int n_beam) { return (n_beam + 2) * kTile; }
-  static constexpr int depth(int n_beam) {
-    const int d = (int)((kMmSmem - kFixed) / (size_t)stage_bytes(n_beam));
+  static constexpr int depth(int n_beam, int ctas) {
+    const size_t room = ctas > 1 ? kMmSmem / ctas - 1024 : kMmSmem;
+    const int d = (int)((room - kFixed) / (size_t)stage_bytes(n_beam));
     return d < kMmMaxD ? d : kMmMaxD;
   }
 };
@@ -190,7 +196,7 @@ __device__ __forceinline__ void pin(uint32_t& x) { asm volatile("" : "+r"(x)); }
 // The XOR that a tensor map's swizzle of `pitch` bytes applies to the 16-byte
 // column of row r (rows `pitch` bytes apart).
 __device__ __forceinline__ int swizzle(int pitch, int r) {
-  return pitch == 128 ? r & 7 : (pitch == 64 ? (r >> 1) & 3 : (r >> 2) & 1);
+  return pitch == 128 ? r & 7 : (pitch == 64 ? (r >> 1) & 3 : (pitch == 32 ? (r >> 2) & 1 : 0));
 }
 
 // One cp.async of kBytes; the barrier's phase completes when every thread's
@@ -204,7 +210,7 @@ __device__ __forceinline__ void mbar_arrive_copies(uint64_t* bar) {
 }
 
 template <class C, bool kTma>
-__global__ void __launch_bounds__(C::kThreads, 1)
+__global__ void __launch_bounds__(C::kThreads, C::kCtas)
 gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const MmArgs g) {
   constexpr int NB = C::NB;
@@ -737,7 +743,8 @@ cudaError_t launch_cfg(const mraid_plan_s* pl, MmArgs& a, bool tma) {
     };
     if (encode(&ma, C::kChA, C::kChA == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                            : C::kChA == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                           : CU_TENSOR_MAP_SWIZZLE_32B) != CUDA_SUCCESS)
+                           : C::kChA == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                           : CU_TENSOR_MAP_SWIZZLE_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
     mb = ma;
     if (C::kChB > 0 && encode(&mb, C::kChB, CU_TENSOR_MAP_SWIZZLE_32B) != CUDA_SUCCESS)
@@ -745,8 +752,10 @@ cudaError_t launch_cfg(const mraid_plan_s* pl, MmArgs& a, bool tma) {
   }
   const int64_t items = (int64_t)a.n_sub * ((p.n_chan + C::kCh - 1) / C::kCh);
   if (items < 1) return cudaSuccess;
-  const int grid = (int)(items < pl->sm_count ? items : pl->sm_count);
-  a.depth = C::depth(a.n_beam);
+  const int ctas = items > pl->sm_count ? C::kCtas : 1;
+  const int64_t slots = (int64_t)pl->sm_count * ctas;
+  const int grid = (int)(items < slots ? items : slots);
+  a.depth = C::depth(a.n_beam, ctas);
   const size_t smem = C::kFixed + (size_t)a.depth * C::stage_bytes(a.n_beam);
   auto kern = tma ? gram_mma_kernel<C, true> : gram_mma_kernel<C, false>;
   cudaError_t e =
@@ -754,6 +763,13 @@ cudaError_t launch_cfg(const mraid_plan_s* pl, MmArgs& a, bool tma) {
   if (e != cudaSuccess) return e;
   kern<<<grid, C::kThreads, smem, pl->stream>>>(ma, mb, a);
   return cudaGetLastError();
+}
+
+// Bytes of a plain copy: 8 or 4 where every row of every beam allows it.
+int copy_bytes(const mraid_plan_s* pl, const void* d_data) {
+  const uint64_t align =
+      (uint64_t)pl->p.n_chan | (uint64_t)pl->beam_stride | (uint64_t)(uintptr_t)d_data;
+  return align % 8 == 0 ? 8 : (align % 4 == 0 ? 4 : 1);
 }
 
 // Time of a launch with work items of `width` channels, in arbitrary units:
@@ -770,20 +786,63 @@ int64_t item_cost(int n_sub, int n_chan, int sm_count, int width, int rate) {
 // ones leave less of the last round over the SMs empty. Sub-integrations of
 // several pieces keep int32 sums of every channel in shared memory:
 // 64-channel items for 16 beams and more, whose sums leave the ring of wider
-// ones too shallow. From 24 beams on 32.
+// ones too shallow. From 24 beams on 32. Blocks of up to 16 channels and more
+// sub-integrations than SMs take 16 (19 beams x 16 channels x 512 samples x 500
+// 39 us, in 32-channel items 61).
 int item_width(const mraid_plan_s* pl, int n_sub) {
   const mraid_params& p = pl->p;
+  const bool lng = p.n_samp_sub > kMmPiece && p.n_samp_sub <= kMmLongMax;
   if (p.n_beam > 23) return 32;
+  if (p.n_chan <= 16 && n_sub > pl->sm_count && !lng) return 16;
   auto cost = [&](int width, int rate) {
     return item_cost(n_sub, p.n_chan, pl->sm_count, width, rate);
   };
   const int64_t c32 = cost(32, 55), c64 = cost(64, 100);
-  const bool lng = p.n_samp_sub > kMmPiece && p.n_samp_sub <= kMmLongMax;
   if (lng && p.n_beam <= 15) return c32 < cost(128, 137) ? 32 : 128;
   if (lng || p.n_beam > 19) return c32 < c64 ? 32 : 64;
   const int wide = p.n_beam <= 15 ? 128 : 96;
   const int64_t cw = p.n_beam <= 15 ? cost(128, 137) : cost(96, 113);
   return c32 < c64 && c32 < cw ? 32 : (cw <= c64 ? wide : 64);
+}
+
+// Microseconds of a call here and on dp4a, from 2 066 timed pairs (2 to 39
+// beams, 1 to 4 096 channels, 8 to 65 536 samples, 1 to 20 000
+// sub-integrations, copies of every kind; within 15 % for most). A stage of 16
+// samples takes an item its time whatever its channels, so a block of few
+// channels pays for 32; dp4a's small blocks share an SM and take the channels
+// there are. At a few blocks per SM it is bound by a chunk's latency. (Its
+// correlation is a second launch, 3 us.) By these figures the slower route is
+// taken in 21 of the pairs by more than 20 %, at the worst by 42 %.
+double mma_us(const mraid_plan_s* pl, const void* d_data) {
+  const mraid_params& p = pl->p;
+  const int N = p.n_beam, width = item_width(pl, p.n_sub);
+  const int64_t items = (int64_t)p.n_sub * ((p.n_chan + width - 1) / width);
+  const int ctas = width > 32 || N > 23 || items <= pl->sm_count ? 1
+                   : (N <= 7 ? 3 : 2) * (width == 16 ? 2 : 1);
+  const int64_t slots = (int64_t)pl->sm_count * ctas;
+  const int kind = copy_bytes(pl, d_data);
+  double stage = N <= 7 ? 0.31 : N <= 15 ? 0.40 : N <= 31 ? 0.51 : 0.69;
+  const bool tail = kind == 1 && p.n_chan % 4 != 0 && p.n_chan <= 32;  // single bytes in every row
+  if (tail) stage = N <= 23 ? 1.1 + 0.13 * N : 1.0 + 0.11 * N;
+  else if (kind == 1) stage = (0.7 + 0.05 * N) * (width == 64 || width == 96 ? 1.4 : 1.0);
+  else if (!gram_mma_bulk(pl, d_data)) stage += 0.33 + (kind == 8 ? 0.007 : 0.012) * N;
+  stage *= width == 32 ? (ctas > 1 ? 1.17 : 1.0) : (width == 64 ? 1.15 : 1.4);
+  const double epilogue = (N <= 7 ? 1.0 : N <= 15 ? 2.3 : N <= 23 ? 3.5 : N <= 31 ? 5.0 : 9.0) *
+                          width / 32 * (width > 32 ? 0.75 : 1.0);
+  const int stages = (p.n_samp_sub + kMmT - 1) / kMmT;
+  return 6.0 + (double)((items + slots - 1) / slots) * (stage * stages + epilogue * ctas);
+}
+double dp4a_us(const mraid_plan_s* pl, const void* d_data) {
+  const mraid_params& p = pl->p;
+  int cpb, tiles;
+  gram_u8_shape(p.n_beam, p.n_chan, &cpb, &tiles);
+  const int tasks = cpb * tiles;
+  const double bytes = cpb % 4 == 0 && copy_bytes(pl, d_data) >= 4 ? 0.0 : p.n_beam * cpb;  // loaded singly
+  const double per_sm = (double)p.n_sub * ((p.n_chan + cpb - 1) / cpb) / pl->sm_count;
+  const double latency = 0.8 + 0.0045 * tasks + 0.025 * bytes;
+  const double issue = per_sm * (0.2 + (p.n_beam < 32 ? 0.006 : 0.0045) * tasks + 0.016 * bytes);
+  const double chunks = (p.n_samp_sub + 31) / 32 * (bytes > 0 && p.n_samp_sub > 2048 ? 1.3 : 1.0);
+  return 9.0 + chunks * (latency > issue ? latency : issue) + per_sm * (0.2 + cpb * (0.03 + 0.0008 * pl->psum));
 }
 
 }  // namespace
@@ -798,21 +857,17 @@ bool gram_mma_bulk(const mraid_plan_s* pl, const void* d_data) {
          encode_fn() != nullptr;
 }
 
-// Few beams by plain copies leave long sub-integrations bound by the length
-// of a stage (0.5-0.7 us, whatever its few products), and dp4a with its many
-// small blocks is the faster one: measured at 1000 channels, 2 beams x 3000
-// samples x 12 0.130 ms against 0.183 here, 7 beams x 3000 x 3 0.123 against
-// 0.134-0.166, but 0.231 against 0.192 at 12 sub-integrations (384 items of 32
-// channels), and 0.031 against 0.024 for 4 beams x 64 x 40. Copies of single
-// bytes are slower on dp4a throughout (1001 channels, 2 beams: 0.332 against
-// 0.326; 36 beams x 1000 samples x 20: 5.7 against 1.15).
+// Narrow blocks, and few beams by plain copies, are faster on dp4a where there
+// are enough of them (measured, dp4a against here): 19 beams x 1 channel x
+// 1024 samples x 2 000 193 us against 505, 7 x 4 x 1024 x 1 000 65 against 127,
+// 13 x 8 x 1024 x 38 40 against 58, 7 beams x 40 channels x 512 x 200 42
+// against 58; but 19 x 16 x 1024 x 250 92 against 50, 19 x 17 x 1024 x 250 454
+// against 237, and from 32 channels on, by bulk copies, never. By the plan's
+// shape, so that ranges of one plan take one route.
 bool gram_mma_takes(const mraid_plan_s* pl, const void* d_data) {
-  const mraid_params& p = pl->p;
   if (!gram_mma_supported(pl)) return false;
-  if (p.n_beam > 7 || p.n_samp_sub < 512 || gram_mma_bulk(pl, d_data)) return true;
-  const bool words =
-      (((uint64_t)p.n_chan | (uint64_t)pl->beam_stride | (uint64_t)(uintptr_t)d_data) & 3) == 0;
-  return !words || (p.n_beam > 2 && (int64_t)p.n_sub * ((p.n_chan + 31) / 32) > pl->sm_count);
+  if (pl->p.n_chan > 16 && gram_mma_bulk(pl, d_data)) return true;
+  return mma_us(pl, d_data) <= dp4a_us(pl, d_data);
 }
 
 bool gram_mma_has_forms(const mraid_plan_s* pl) {
@@ -832,8 +887,7 @@ cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int s
   MmArgs a;
   a.data = d_data;
   a.beam_stride = pl->beam_stride;
-  const uint64_t align = (uint64_t)p.n_chan | (uint64_t)pl->beam_stride | (uint64_t)(uintptr_t)d_data;
-  a.vec = align % 8 == 0 ? 8 : (align % 4 == 0 ? 4 : 1);
+  a.vec = copy_bytes(pl, d_data);
   a.data_end = d_data + (int64_t)(p.n_beam - 1) * pl->beam_stride +
                (int64_t)(sub0 + n_sub) * p.n_samp_sub * p.n_chan;
   a.n_beam = p.n_beam;
@@ -869,19 +923,23 @@ cudaError_t launch_gram_mma(const mraid_plan_s* pl, const uint8_t* d_data, int s
   if (p.n_beam > 31) return launch_cfg<MmCfg<5, false, 32, 0, 4>>(pl, a, tma);
   if (p.n_beam > 23) return launch_cfg<MmCfg<4, false, 32, 0, 4>>(pl, a, tma);
   if (p.n_beam <= 7)
-    return pick == 32   ? launch_cfg<MmCfg<1, false, 32, 0>>(pl, a, tma)
+    return pick == 16   ? launch_cfg<MmCfg<1, false, 16, 0>>(pl, a, tma)
+           : pick == 32 ? launch_cfg<MmCfg<1, false, 32, 0>>(pl, a, tma)
            : pick == 64 ? launch_cfg<MmCfg<1, false, 64, 0>>(pl, a, tma)
                         : launch_cfg<MmCfg<1, false, 128, 0>>(pl, a, tma);
   if (p.n_beam <= 15)
-    return pick == 32   ? launch_cfg<MmCfg<2, false, 32, 0>>(pl, a, tma)
+    return pick == 16   ? launch_cfg<MmCfg<2, false, 16, 0>>(pl, a, tma)
+           : pick == 32 ? launch_cfg<MmCfg<2, false, 32, 0>>(pl, a, tma)
            : pick == 64 ? launch_cfg<MmCfg<2, false, 64, 0>>(pl, a, tma)
                         : launch_cfg<MmCfg<2, false, 128, 0>>(pl, a, tma);
   if (p.n_beam <= 19)
-    return pick == 32   ? launch_cfg<MmCfg<3, true, 32, 0>>(pl, a, tma)
+    return pick == 16   ? launch_cfg<MmCfg<3, true, 16, 0>>(pl, a, tma)
+           : pick == 32 ? launch_cfg<MmCfg<3, true, 32, 0>>(pl, a, tma)
            : pick == 64 ? launch_cfg<MmCfg<3, true, 64, 0>>(pl, a, tma)
                         : launch_cfg<MmCfg<3, true, 64, 32>>(pl, a, tma);
-  return pick == 32 ? launch_cfg<MmCfg<3, false, 32, 0>>(pl, a, tma)
-                    : launch_cfg<MmCfg<3, false, 64, 0>>(pl, a, tma);
+  return pick == 16   ? launch_cfg<MmCfg<3, false, 16, 0>>(pl, a, tma)
+         : pick == 32 ? launch_cfg<MmCfg<3, false, 32, 0>>(pl, a, tma)
+                      : launch_cfg<MmCfg<3, false, 64, 0>>(pl, a, tma);
 }
 
 }  // namespace mraid

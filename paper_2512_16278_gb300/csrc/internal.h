@@ -170,6 +170,8 @@ mraid_status cuda_fail(cudaError_t e, const char* what);
 // by cell relative to sub0 (cell = (sub - sub0) * n_chan + chan).
 cudaError_t launch_gram_u8(const mraid_plan_s* pl, const uint8_t* d_data,
                            int sub0, int n_sub, int64_t* d_sums);
+// channels per block and 4 x 4 output tiles of the dp4a Gram
+void gram_u8_shape(int n_beam, int n_chan, int* cpb, int* tiles);
 // float32 samples: correlation on CUDA cores (d_corr relative to sub0)
 cudaError_t launch_gram_f32(const mraid_plan_s* pl, const float* d_data, int sub0, int n_sub,
                             float* d_corr);
