@@ -1,4 +1,5 @@
-// gram_tcl.cu - exact augmented Gram sums of 8-bit data for 40..127 beams
+// gram_tcl.cu - exact augmented Gram sums of 8-bit data for 40..127 beams, and
+// for 32..39 where few long sub-integrations make it the faster one,
 // on the tensor cores, channels kept apart by rows.
 //
 // Section 3.2, Eq. 1, for the larger (phased-array-feed) receivers. The
@@ -483,9 +484,22 @@ int l_channels(int n_beam, int* n_u8_out) {
 
 }  // namespace
 
+// From 32 to 39 beams the register-fragment Gram is the faster one where its
+// 32-channel items fill the SMs, but a few long sub-integrations leave both
+// with the length of one item's chain, and 8 channels per pass are the shorter
+// one (measured against it: 36 beams x 64 channels x 65 536 samples 1.70 ms
+// against 2.82, x 4 096 0.136 against 0.191, 256 x 2 048 x 4 0.085 against
+// 0.103; x 1 024 0.058 against 0.058; with 256 channels x 2 048 x 8, two rounds
+// of these passes, 0.143 against 0.105).
+bool gram_tcl_takes(const mraid_plan_s* pl, const void* d_data) {
+  const mraid_params& p = pl->p;
+  return p.n_beam <= 39 && p.n_samp_sub >= 2048 &&
+         2 * (int64_t)p.n_sub * (p.n_chan / 16) <= pl->sm_count && gram_tcl_supported(pl, d_data);
+}
+
 bool gram_tcl_supported(const mraid_plan_s* pl, const void* d_data) {
   const mraid_params& p = pl->p;
-  return p.bit_depth == 8 && p.n_beam >= 40 && p.n_beam + 1 <= 128 &&
+  return p.bit_depth == 8 && p.n_beam >= 32 && p.n_beam + 1 <= 128 &&
          p.n_samp_sub % kLT == 0 && p.n_samp_sub <= 65536 && p.n_chan % 16 == 0 &&
          pl->beam_stride % 16 == 0 && (reinterpret_cast<uintptr_t>(d_data) & 15) == 0 &&
          (int64_t)p.n_sub * p.n_samp_sub <= 2147483647ll && l_channels(p.n_beam, nullptr) > 0 &&

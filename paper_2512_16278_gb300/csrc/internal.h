@@ -184,10 +184,12 @@ constexpr int kTcVariants = 10;  // 8-bit tensor-core Gram ids: 0, 1 and aliases
 constexpr int kEigVariants = 6;  // register eigensolvers (see eig_variant)
 // float32 samples on the tensor cores (split-bf16 products, gram_tc.cu):
 // correlation only, d_corr relative to sub0
-// Tensor-core Gram for 40..127 beams, one or two channels per MMA (gram_tcl.cu):
+// Tensor-core Gram for 32..127 beams, one or two channels per MMA (gram_tcl.cu):
 // int64 sums [cell][P] of sub-integrations [sub0, sub0 + n_sub), cells
 // relative to sub0.
 bool gram_tcl_supported(const mraid_plan_s* pl, const void* d_data);
+// 32..39 beams: supported, and faster than gram_mma for the plan's shape
+bool gram_tcl_takes(const mraid_plan_s* pl, const void* d_data);
 cudaError_t launch_gram_tcl(const mraid_plan_s* pl, const uint8_t* d_data, int sub0, int n_sub,
                             int64_t* d_sums);
 // gram_mma.cu: 8-bit Gram for up to 39 beams, any layout, fused with the

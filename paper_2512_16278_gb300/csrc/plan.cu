@@ -224,7 +224,7 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
     }
     return MRAID_OK;
   }
-  const bool mma = !pl->force_dp4a && gram_mma_takes(pl, d_data);
+  const bool mma = !pl->force_dp4a && gram_mma_takes(pl, d_data) && !gram_tcl_takes(pl, d_data);
   // profiled by the way the samples come: "gram_tc" for bulk tensor copies
   // ("gram_tcl" above 23 beams)
   const int mma_id = !(mma && gram_mma_bulk(pl, d_data)) ? K_GRAM
@@ -247,7 +247,8 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
                                launch_gram_mma(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
                                                sums, nullptr));
     if (e != cudaSuccess) return cuda_fail(e, "gram_mma launch");
-  } else if (!pl->force_dp4a && gram_tcl_supported(pl, d_data)) {
+  } else if (!pl->force_dp4a &&
+             (pl->p.n_beam < 40 ? gram_tcl_takes(pl, d_data) : gram_tcl_supported(pl, d_data))) {
     cudaError_t e = MRAID_PROF(pl, K_GRAM_TCL,
                                launch_gram_tcl(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
                                                sums));
@@ -789,7 +790,7 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
   // that are aliases too.
   const bool mma = gram_mma_supported(pl);
   const bool tc = pl->p.bit_depth == 32 ? gram_tc_f32_supported(pl, d_data)
-                  : mma                 ? gram_mma_takes(pl, d_data)
+                  : mma                 ? gram_mma_takes(pl, d_data) || gram_tcl_takes(pl, d_data)
                                         : gram_tcl_supported(pl, d_data);
   const int last = tc ? (mma && gram_mma_has_forms(pl) ? 1 : 0) : -1;
   float ms[3] = {};  // of ids -1, 0, 1

@@ -1,0 +1,54 @@
+"""32 to 39 beams, few long sub-integrations (needs a GPU): the Gram with
+channels kept apart by rows takes them, with the sums of the CUDA-core Gram
+bit for bit at the rule's edges, and at the speed of 40 beams."""
+import pytest
+
+from gpu_util import lib
+
+pytestmark = pytest.mark.gpu
+
+
+def block(n_beam, n_chan, n_s, n_sub):
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n_beam + n_chan)
+    return torch.randint(0, 256, (n_beam, n_sub * n_s, n_chan), dtype=torch.uint8, device="cuda", generator=g)
+
+
+@pytest.mark.parametrize("n_beam", [32, 36, 39])
+@pytest.mark.parametrize("n_chan,n_s,n_sub", [
+    (16, 2048, 1), (16, 65536, 2), (608, 2048, 2), (624, 2048, 2), (32, 2080, 3), (33, 4096, 1), (64, 3072, 4),
+])
+def test_same_sums_as_the_cuda_cores(n_beam, n_chan, n_s, n_sub):
+    import torch
+    m = lib()
+    d = block(n_beam, n_chan, n_s, n_sub)
+    got = {}
+    for variant in (0, -1):
+        with m.Plan(n_beam, n_chan, n_s, n_sub) as plan:
+            m.mraid_set_variant(plan.handle, variant)
+            got[variant] = plan.ccm(d)
+            plan.sync()
+    assert torch.equal(got[0][0], got[-1][0])
+    assert (got[0][1] - got[-1][1]).abs().max() <= 2e-6
+
+
+def test_as_fast_as_forty_beams():
+    import torch
+    m = lib()
+    n_chan, n_s, n_sub = 64, 16384, 1
+    times = []
+    for n_beam in (36, 40):
+        d = block(n_beam, n_chan, n_s, n_sub)
+        with m.Plan(n_beam, n_chan, n_s, n_sub) as plan:
+            corr = torch.empty(plan.n_cells, n_beam * (n_beam + 1) // 2, device="cuda")
+            runs = []
+            for _ in range(8):
+                e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                e0.record()
+                m.mraid_ccm(plan.handle, d, None, corr)
+                e1.record()
+                torch.cuda.synchronize()
+                runs.append(e0.elapsed_time(e1))
+            times.append(sorted(runs[1:])[3])
+    assert times[0] < 1.2 * times[1], times
