@@ -463,28 +463,45 @@ __global__ void ccm_bandpass_kernel(const int64_t* __restrict__ sums, int64_t n_
 
 }  // namespace
 
-// CTAs per spectrum: two for long spectra that leave SMs idle, and as many as
-// it takes for the arrays to fit shared memory. Measured on GB300, us a call
-// of 5 to 6 solves with 1 / 2 / 4 / 8 CTAs: 38 spectra of 4096 channels 904 /
-// 696 / 994 / 1290, 190 spectra 1650 / 1845 / 2793 / 5303, 38 spectra of 1000
-// channels 420 / 431 / 649 / 1093 (the cluster's barriers and the serial top
-// outweigh the share of the FP64 work).
-int arpls_ctas(int n, int n_sys, int sm_count) {
-  const int m = cr_rows(n);
-  int k = m >= 1024 && (int64_t)n_sys * 2 <= sm_count ? 2 : 1;
-  while (k < kArMaxCtas && (size_t)kCrArrays * (m / k) * sizeof(double) > kArSmem) k *= 2;
-  return k;
-}
-// Shared memory of one of k CTAs; 0: the arrays live in global memory (k = 1)
+// Shared memory of one of k CTAs; 0: the arrays do not fit
 size_t arpls_smem_bytes(int n, int k) {
   const size_t b = (size_t)kCrArrays * (cr_rows(n) / k) * sizeof(double);
   return b <= kArSmem ? b : 0;
 }
 
-size_t arpls_work_doubles(int n, int n_sys) {
-  // the weights always; the reduction arrays when they are not in shared memory
-  return (size_t)2 * n * n_sys +
-         (arpls_smem_bytes(n, kArMaxCtas) ? 0 : (size_t)kCrArrays * cr_rows(n) * n_sys);
+// CTAs per spectrum with the arrays in shared memory: two for long spectra
+// that leave SMs idle, and as many as it takes for the arrays to fit; 0 where
+// eight do not. Measured on GB300, us a call of 5 to 6 solves with 1 / 2 / 4 /
+// 8 CTAs: 38 spectra of 4096 channels 904 / 696 / 994 / 1290, 190 spectra 1650
+// / 1845 / 2793 / 5303, 38 spectra of 1000 channels 420 / 431 / 649 / 1093 (the
+// cluster's barriers and the serial top outweigh the share of the FP64 work).
+int arpls_ctas(int n, int n_sys, int sm_count) {
+  const int m = cr_rows(n);
+  int k = m >= 1024 && (int64_t)n_sys * 2 <= sm_count ? 2 : 1;
+  while (k < kArMaxCtas && !arpls_smem_bytes(n, k)) k *= 2;
+  return arpls_smem_bytes(n, k) ? k : 0;
+}
+
+// True where one CTA per spectrum on global memory is the faster way: many
+// spectra that need a cluster for their arrays. A cluster of 2 / 4 / 8 is 1.67 /
+// 3.05 / 5.4 times as fast as such a CTA, but 152 SMs hold 76 / 34 / 15 of them
+// at a time (not every SM has neighbours left for a cluster). Measured, clusters
+// against global memory: 760 spectra of 8192 channels 8.70 ms against 6.84, 190
+// 2.51 against 2.79; 760 of 16 384 18.7 against 13.0, 38 1.71 against 2.52; 400
+// of 32 768 23.5 against 16.0, 38 2.62 against 4.76.
+bool arpls_on_global(const mraid_plan_s* pl, int n, int n_sys) {
+  const int sm_count = pl->sm_count, k = arpls_ctas(n, n_sys, sm_count);
+  if (k == 0) return true;
+  if (arpls_smem_bytes(n, 1) || pl->ar_work_short) return false;
+  const double gain = k == 2 ? 1.67 : (k == 4 ? 3.05 : 5.4);
+  const int held = k == 2 ? sm_count / 2 : (k == 4 ? sm_count * 9 / 40 : sm_count / 10);
+  const int64_t rounds = ((int64_t)n_sys + held - 1) / held;
+  return (double)(((int64_t)n_sys + sm_count - 1) / sm_count) * gain < (double)rounds;
+}
+
+// the weights always; the reduction arrays when they are not in shared memory
+size_t arpls_work_doubles(int n, int n_sys, bool on_global) {
+  return (size_t)2 * n * n_sys + (on_global ? (size_t)kCrArrays * cr_rows(n) * n_sys : 0);
 }
 
 cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, int n, double lam,
@@ -503,10 +520,10 @@ cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, i
   g.itermax = itermax;
   g.lam = lam;
   g.ratio = ratio;
-  int k = arpls_ctas(n, n_sys, pl->sm_count);
-  const size_t smem = arpls_smem_bytes(n, k);
-  if (!smem) k = 1;  // one CTA per spectrum on global memory
-  g.in_smem = smem ? 1 : 0;
+  const bool on_global = arpls_on_global(pl, n, n_sys);
+  const int k = on_global ? 1 : arpls_ctas(n, n_sys, pl->sm_count);
+  const size_t smem = on_global ? 0 : arpls_smem_bytes(n, k);
+  g.in_smem = on_global ? 0 : 1;
   cudaError_t e = cudaFuncSetAttribute(arpls_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
@@ -564,14 +581,22 @@ mraid_status check_bandpass_params(const mraid_bandpass_params* bp) {
   return MRAID_OK;
 }
 
-// ArPLS arrays in global memory for spectra too long for shared memory
+// ArPLS weights, and the arrays of spectra that are solved on global memory; if
+// these do not fit it and clusters can do without, the weights alone, and the
+// plan stays on clusters
 mraid_status ensure_arpls_work(mraid_plan_s* pl, int n, int n_sys) {
-  const size_t need = arpls_work_doubles(n, n_sys);
+  size_t need = arpls_work_doubles(n, n_sys, arpls_on_global(pl, n, n_sys));
   if (need <= pl->ar_work_elems) return MRAID_OK;
   cudaFree(pl->ar_work);
   pl->ar_work = nullptr;
   pl->ar_work_elems = 0;
   cudaError_t e = cudaMalloc(&pl->ar_work, need * sizeof(double));
+  if (e != cudaSuccess && arpls_ctas(n, n_sys, pl->sm_count) > 0) {
+    cudaGetLastError();
+    pl->ar_work_short = true;
+    need = arpls_work_doubles(n, n_sys, false);
+    e = cudaMalloc(&pl->ar_work, need * sizeof(double));
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cuda_fail(e, "arpls work allocation");

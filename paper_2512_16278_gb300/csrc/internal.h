@@ -121,6 +121,7 @@ struct mraid_plan_s {
   size_t bp_sys = 0;
   double* ar_work = nullptr;
   size_t ar_work_elems = 0;
+  bool ar_work_short = false;  // the arrays of the global-memory route did not fit once
   // two polarisations: Gram sums of the 2N stacked blocks where the tensor
   // cores do not take the block; pol_cells counts its int64 elements
   int64_t* pol_sums = nullptr;
@@ -244,8 +245,9 @@ cudaError_t launch_flag(mraid_plan_s* pl, const float* d_stat, uint8_t* d_flags,
                         int64_t n_cells = -1, mraid_flag_info* d_info = nullptr);
 // bandpass.cu: ArPLS baselines of n_sys spectra of n points ([sys][n]
 // FP64; d_zf an optional float copy, d_iters solves per spectrum or -1);
-// d_work holds arpls_work_doubles(n, n_sys) doubles when that is nonzero
-size_t arpls_work_doubles(int n, int n_sys);
+// d_work holds arpls_work_doubles(n, n_sys, arpls_on_global(pl, n, n_sys)) doubles
+bool arpls_on_global(const mraid_plan_s* pl, int n, int n_sys);
+size_t arpls_work_doubles(int n, int n_sys, bool on_global);
 cudaError_t launch_arpls(const mraid_plan_s* pl, const double* d_y, int n_sys, int n, double lam,
                          double ratio, int itermax, double* d_z, float* d_zf, int32_t* d_iters,
                          double* d_work);
