@@ -468,7 +468,11 @@ void mraid_destroy(mraid_plan_t plan);
  * launches with a pair of CUDA events on its stream; mraid_sync folds the
  * elapsed times into per-kernel totals. mraid_profile_read copies up to max
  * records (name, launches, total milliseconds) into out and sets *n to the
- * number of kernels seen; mraid_profile_reset clears the totals. */
+ * number of kernels seen; mraid_profile_reset clears the totals. The Gram of
+ * 8-bit samples has three names, kept over its kernels: "gram_tc" (bulk tensor
+ * copies, up to 23 beams, and two polarisations), "gram_tcl" (bulk tensor
+ * copies, 24 beams and more) and "gram_u8" (plain copies, on the tensor cores
+ * or not); mraid_gram_kernel tells the kernel. */
 typedef struct {
   char name[32];
   int64_t launches;
@@ -479,6 +483,14 @@ mraid_status mraid_profile_enable(mraid_plan_t plan, int32_t enable);
 mraid_status mraid_profile_read(mraid_plan_t plan, mraid_kernel_time* out, int32_t max,
                                 int32_t* n);
 mraid_status mraid_profile_reset(mraid_plan_t plan);
+
+/* The kernel that forms the Gram of a block at d_data (by the plan's shape and
+ * variant, and the buffer's alignment; nothing is read from it), as a static
+ * string: "gram_mma" (tensor cores, register fragments; 8-bit, up to 39 beams),
+ * "gram_mma, plain copies" (the same for layouts that no tensor map takes),
+ * "gram_tcl" (tensor cores, tcgen05; 32 to 127 beams), "gram_u8" (CUDA cores),
+ * "gram_tc_f32" and "gram_f32" (float32 samples); "" for a NULL plan. */
+const char* mraid_gram_kernel(mraid_plan_t plan, const void* d_data);
 
 /* Static strings. mraid_last_error describes the last failure in this
  * thread (empty if none). */

@@ -21,7 +21,7 @@ __all__ = [
     "mraid_default_params", "mraid_validate", "mraid_plan", "mraid_ccm", "mraid_eig",
     "mraid_flag", "mraid_run", "mraid_run_host", "mraid_sync", "mraid_query",
     "mraid_destroy", "mraid_status_string", "mraid_last_error", "mraid_abi_version",
-    "mraid_profile_enable", "mraid_profile_read", "mraid_profile_reset", "mraid_ccm_noalloc",
+    "mraid_profile_enable", "mraid_profile_read", "mraid_profile_reset", "mraid_gram_kernel", "mraid_ccm_noalloc",
     "mraid_batch_plan", "mraid_batch_run", "mraid_batch_sync", "mraid_batch_graph_stats",
     "mraid_batch_packing",
     "mraid_batch_destroy", "UnitIO", "Batch", "mraid_serve_open", "mraid_serve_submit",
@@ -166,6 +166,7 @@ def load():
         "mraid_serve_close": (None, [vp]),
         "mraid_autotune": (ctypes.c_int, [vp, vp, i32, ctypes.POINTER(i32), ctypes.POINTER(i32),
                                           ctypes.c_char_p, i32]),
+        "mraid_gram_kernel": (ctypes.c_char_p, [vp, vp]),
         "mraid_set_variant": (ctypes.c_int, [vp, i32]),
         "mraid_set_eig_variant": (ctypes.c_int, [vp, i32]),
         "mraid_set_wait_limit": (ctypes.c_int, [vp, ctypes.c_int64]),
@@ -438,6 +439,11 @@ def mraid_autotune(plan: int, d_data, reps: int = 3):
 def mraid_refine(plan: int, d_q1, d_flags, d_beam_bits, d_mu_sigma=None):
     _check(load().mraid_refine(plan, _ptr(d_q1), _ptr(d_flags), _ptr(d_beam_bits),
                                _ptr(d_mu_sigma)), "mraid_refine")
+
+
+def mraid_gram_kernel(plan: int, d_data) -> str:
+    """Name of the kernel that forms the Gram of a block at d_data."""
+    return load().mraid_gram_kernel(plan, _ptr(d_data)).decode()
 
 
 def mraid_set_variant(plan: int, variant: int):

@@ -198,6 +198,17 @@ mraid_status check_plan(mraid_plan_t pl) {
   return MRAID_OK;
 }
 
+// The kernel that forms the 8-bit Gram of a plan's block.
+namespace {
+enum GramRoute { R_DP4A, R_MMA, R_TCL };
+GramRoute gram_route(const mraid_plan_s* pl, const void* d_data) {
+  if (pl->force_dp4a) return R_DP4A;
+  if (gram_mma_supported(pl))
+    return gram_tcl_takes(pl, d_data) ? R_TCL : (gram_mma_takes(pl, d_data) ? R_MMA : R_DP4A);
+  return gram_tcl_supported(pl, d_data) ? R_TCL : R_DP4A;
+}
+}  // namespace
+
 // Gram sums + correlation of sub-integrations [sub0, sub0+n_sub) of d_data;
 // d_sums / d_corr are indexed by cell relative to sub0.
 mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub, int64_t* d_sums,
@@ -224,9 +235,11 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
     }
     return MRAID_OK;
   }
-  const bool mma = !pl->force_dp4a && gram_mma_takes(pl, d_data) && !gram_tcl_takes(pl, d_data);
+  const GramRoute route = gram_route(pl, d_data);
+  const bool mma = route == R_MMA;
   // profiled by the way the samples come: "gram_tc" for bulk tensor copies
-  // ("gram_tcl" above 23 beams)
+  // ("gram_tcl" above 23 beams), "gram_u8" for plain ones; mraid_gram_kernel
+  // names the kernel
   const int mma_id = !(mma && gram_mma_bulk(pl, d_data)) ? K_GRAM
                      : pl->p.n_beam <= 23                ? K_GRAM_TC
                                                          : K_GRAM_TCL;
@@ -247,8 +260,7 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
                                launch_gram_mma(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
                                                sums, nullptr));
     if (e != cudaSuccess) return cuda_fail(e, "gram_mma launch");
-  } else if (!pl->force_dp4a &&
-             (pl->p.n_beam < 40 ? gram_tcl_takes(pl, d_data) : gram_tcl_supported(pl, d_data))) {
+  } else if (route == R_TCL) {
     cudaError_t e = MRAID_PROF(pl, K_GRAM_TCL,
                                launch_gram_tcl(pl, static_cast<const uint8_t*>(d_data), sub0, n_sub,
                                                sums));
@@ -789,9 +801,9 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
   // not where the rule takes the CUDA cores anyway. The report has the ids
   // that are aliases too.
   const bool mma = gram_mma_supported(pl);
+  pl->force_dp4a = false;
   const bool tc = pl->p.bit_depth == 32 ? gram_tc_f32_supported(pl, d_data)
-                  : mma                 ? gram_mma_takes(pl, d_data) || gram_tcl_takes(pl, d_data)
-                                        : gram_tcl_supported(pl, d_data);
+                                        : gram_route(pl, d_data) != R_DP4A;
   const int last = tc ? (mma && gram_mma_has_forms(pl) ? 1 : 0) : -1;
   float ms[3] = {};  // of ids -1, 0, 1
   for (int v = -1; v <= last && st == MRAID_OK; ++v) {
@@ -852,6 +864,17 @@ mraid_status mraid_autotune(mraid_plan_t pl, const void* d_data, int32_t reps, i
   *gram_choice = best_g;
   *eig_choice = best_e;
   return MRAID_OK;
+}
+
+const char* mraid_gram_kernel(mraid_plan_t pl, const void* d_data) {
+  if (check_plan(pl) != MRAID_OK) return "";
+  if (pl->p.bit_depth == 32)
+    return !pl->force_dp4a && gram_tc_f32_supported(pl, d_data) ? "gram_tc_f32" : "gram_f32";
+  switch (gram_route(pl, d_data)) {
+    case R_MMA: return gram_mma_bulk(pl, d_data) ? "gram_mma" : "gram_mma, plain copies";
+    case R_TCL: return "gram_tcl";
+    default: return "gram_u8";
+  }
 }
 
 mraid_status mraid_profile_enable(mraid_plan_t pl, int32_t enable) {
