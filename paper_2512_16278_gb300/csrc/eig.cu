@@ -850,8 +850,11 @@ eig_tri_kernel(const float* __restrict__ corr, int64_t n_cells, float* __restric
 // beams without eigenvalues 60 -> 27 us, the seven timescales (301 056 cells)
 // 2.26 -> 1.96 ms per call; the statistic's error against 64 bits falls from
 // 5e-6 to 4e-7 there (the QR's deflation bound no longer enters it). With
-// eigenvalues and no q1 the Newton loop costs 5 % (155 648 cells of 13 beams
-// 20 us), so that the statistic is the same bits whatever else is asked for.
+// eigenvalues and no q1 the QR kernel would find lambda_1 too; the Newton loop
+// runs all the same, so that the statistic is the same bits whatever else is
+// asked for (819 200 cells of 19 beams 774 -> 1 001 us, of 13 beams 404 -> 469;
+// run in the QR kernel 946 and 470, but its registers cost the calls with q1 2
+// %).
 // Newton's steps shrink by 1 - 1/m at an m-fold lambda_1: the bound lets an
 // 18-fold one converge to 1e-7 (282 steps); a simple one takes about ten.
 constexpr int kNewtonMax = 400;

@@ -258,18 +258,19 @@ __global__ void __launch_bounds__(kFlagThreads) flag_kernel(FlagArgs f) {
 
 // ---------------------------------------------------------------------------
 // The same iteration on one cluster. What bounds it is latency: a pass costs
-// its cells' issue (about 7 instructions a cell) plus one cluster barrier,
+// its cells' issue (about 8 instructions a cell) plus one cluster barrier,
 // where the cooperative kernel pays a grid barrier and a trip of the partial
-// sums through L2. Measured on GB300 (5 to 7 fits): 1 024 cells 67 -> 15 us,
-// 16 384 67 -> 26, 77 824 86 -> 34, 409 600 93 -> 49, 819 200 101 -> 69; past
-// 868 352 cells (16 CTAs) the cooperative kernel, 102 us.
+// sums through L2. Measured on GB300 (call to call, 4 to 9 fits; cooperative
+// kernel, this one): 1 024 cells 62 and 24 us, 16 384 77 and 38, 77 824 78-88
+// and 38-40, 409 600 107-114 and 63-66, 819 200 112-124 and 87; past 868 352
+// cells (16 CTAs) the cooperative kernel, 113.
 //
 // Sums are taken about a pivot (the last fit's mean; for the first fit the
 // mean of the block's first cells): four cells in FP32, then two floats per
 // moment (value and rounding error) through a fixed tree over lanes, warps and
 // CTAs, the same bits in every CTA. FP64 sums would cost more than the rest of
 // a pass; the fit itself is FP64. The cells' own roundings leave the variance
-// s2 / n - m^2 (m the mean's distance from the pivot) an error of 1e-7 s2 / n at
+// s2 / n - m^2 (m the mean's distance from the pivot) an error of 4e-7 s2 / n at
 // most, so it is only used where it is at least a tenth of s2 / n. Where it is
 // less (the last threshold took out cells that had moved the mean by more than
 // three deviations, or the first cells were unlike the rest) the sums are taken

@@ -26,7 +26,8 @@
 //
 // Layout: a work item is one sub-integration x 32, 64, 96 or 128 channels
 // (4, 8, 12 or 16 warps, as many as the accumulators leave registers for; 32
-// channels and 8 warps from 24 beams on);
+// channels and 8 warps from 24 beams on; 16 channels and 2 warps for narrow
+// blocks; items of 4 warps and fewer share an SM);
 // stages of 16 samples x all beams come by TMA with a swizzle under which a
 // warp's 8-byte loads meet two-way conflicts at most, into a ring as deep as
 // shared memory allows; the warps take turns to issue the copies. Wide rows
@@ -600,40 +601,42 @@ gram_mma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (nu <= 0) break;
         __syncwarp();
         if constexpr (!C::kLong && NB <= 3) {
+          // the same as stage_out for these blocks, written out: with stage_out here
+          // too the kernels of up to 23 beams were 4 to 5 % slower
 #pragma unroll
-        for (int gr = 0; gr < C::kCW / kMmEpi; ++gr) {
-          if (gr * kMmEpi != c0) continue;
+          for (int gr = 0; gr < C::kCW / kMmEpi; ++gr) {
+            if (gr * kMmEpi != c0) continue;
 #pragma unroll
-          for (int u = 0; u < kMmEpi; ++u) {
-            const int c = gr * kMmEpi + u;
-            float* sg = reinterpret_cast<float*>(s->g[warp][u]);
-            auto put = [&](int at, const float* d) {
-              *reinterpret_cast<float2*>(sg + at) = make_float2(d[0], d[1]);
-            };
-            const int e = g8 * 8 + 2 * t;
-            if constexpr (NB == 1) {
-              put(e, acc[c][0] + 2 * (c & 1));
-            } else {
-              put(e, acc[c][0]);            // block 0 x 0
-              put(64 + e, acc[c][1]);       // 0 x 1
-              put(128 + e, acc[c][1] + 2);  // 1 x 1
-              if constexpr (NB == 3 && !kHalf) {
-                put(192 + e, acc[c][2]);
-                put(256 + e, acc[c][2] + 2);
-                put(320 + e, acc[c][3] + 2 * (c & 1));
-              }
-              if constexpr (kHalf) {
-                if ((t >> 1) == (c & 1)) {  // this channel's four of the eight columns
-                  const int e4 = g8 * 4 + 2 * (t & 1);
-                  put(192 + e4, acc2[c / 2][0]);
-                  put(224 + e4, acc2[c / 2][0] + 2);
-                  if ((g8 >> 2) == (c & 1))
-                    put(256 + (g8 & 3) * 4 + 2 * (t & 1), acc2[c / 2][1] + ((c / 2) & 1 ? 2 : 0));
+            for (int u = 0; u < kMmEpi; ++u) {
+              const int c = gr * kMmEpi + u;
+              float* sg = reinterpret_cast<float*>(s->g[warp][u]);
+              auto put = [&](int at, const float* d) {
+                *reinterpret_cast<float2*>(sg + at) = make_float2(d[0], d[1]);
+              };
+              const int e = g8 * 8 + 2 * t;
+              if constexpr (NB == 1) {
+                put(e, acc[c][0] + 2 * (c & 1));
+              } else {
+                put(e, acc[c][0]);            // block 0 x 0
+                put(64 + e, acc[c][1]);       // 0 x 1
+                put(128 + e, acc[c][1] + 2);  // 1 x 1
+                if constexpr (NB == 3 && !kHalf) {
+                  put(192 + e, acc[c][2]);
+                  put(256 + e, acc[c][2] + 2);
+                  put(320 + e, acc[c][3] + 2 * (c & 1));
+                }
+                if constexpr (kHalf) {
+                  if ((t >> 1) == (c & 1)) {  // this channel's four of the eight columns
+                    const int e4 = g8 * 4 + 2 * (t & 1);
+                    put(192 + e4, acc2[c / 2][0]);
+                    put(224 + e4, acc2[c / 2][0] + 2);
+                    if ((g8 >> 2) == (c & 1))
+                      put(256 + (g8 & 3) * 4 + 2 * (t & 1), acc2[c / 2][1] + ((c / 2) & 1 ? 2 : 0));
+                  }
                 }
               }
             }
           }
-        }
         } else if constexpr (!C::kLong) {
           // registers cannot be indexed: the staging of each group is its own code
           static_loop<C::kCW / kMmEpi>([&](auto gr) {
