@@ -58,6 +58,7 @@ struct TcArgs {
   int R;    // slots per group: N + 1
   int R2;   // slots 16..N per group (0 if N + 1 <= 16)
   int rb;   // slots in B of the first MMAs (R rounded up to even)
+  unsigned* progress;  // times that CTAs came to a step (zeroed before the launch)
   int64_t* sums;
   float* corr;
   unsigned long long* degenerate;
@@ -123,6 +124,32 @@ __host__ __device__ constexpr size_t smem_bytes(int n_beam, int n_u8) {
          (size_t)n_u8 * u8_stage_size(n_beam) + sizeof(Smem);
 }
 
+// The CTAs of a launch are kept in step, because neighbours read 16 bytes each
+// of the same lines: once they drift apart by more than L2 holds, every line
+// comes from memory several times, and nothing brings them together again.
+// Without it 13 beams x 4096 channels x 1024 samples x 200 took 6.1 to 15 ms
+// from one call to the next, and 19 beams 8.1 to 17 by the slightest change of
+// the code; in step 6.10 and 8.18 (7 beams 7.0 -> 5.1). A CTA may be one step of
+// kStep stages ahead of the last one (steps of 8 and 16 stages measured the
+// same); the counter is read while a stage's copy is under way. Only the time
+// depends on it: the wait for a CTA that has not started, or has left, ends
+// after kStepNs, and the waiting one goes on alone.
+constexpr int kStep = 4;                       // stages
+constexpr unsigned long long kStepNs = 20000;  // longest wait for the others
+
+// Counts this CTA's coming to a step, and waits, if asked to, until the count
+// is `all`: false if it did not get there in time.
+__device__ __forceinline__ bool all_in_step(unsigned* progress, unsigned all, bool wait) {
+  atomicAdd(progress, 1u);
+  if (!wait) return false;
+  const unsigned long long t0 = gtimer();
+  while (*(volatile unsigned*)progress < all) {
+    if (gtimer() - t0 > kStepNs) return false;
+    __nanosleep(32);
+  }
+  return true;
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
   const int kF16StageBytes = (int)f16_stage_bytes(g.n_beam);
@@ -132,7 +159,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
   const int kNU = g.n_u8;
   unsigned char* f16 = base;                                   // kNF stages
   unsigned char* u8 = f16 + (size_t)kNF * kF16StageBytes;      // kNU stages
-  const int u8_stage_bytes = (int)u8_stage_size(g.n_beam);
+  const int u8_stage_bytes = 2 * g.n_beam * kT * kBoxCh;
   Smem* s = reinterpret_cast<Smem*>(u8 + (size_t)kNU * u8_stage_bytes);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -180,7 +207,9 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
   if (warp == 0) {
     // ------------------------------------------------------------ TMA
     if (lane == 0) {
-      uint32_t cnt = 0;
+      uint32_t cnt = 0, steps = 0;
+      const int64_t whole = items / gridDim.x * gridDim.x;  // items of rounds that every CTA has
+      bool in_step = true;
       long long withheld = -1;
       bool ok = true;
       for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
@@ -199,6 +228,11 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
           mbar_expect_tx(&s->u8_full[slot], (uint32_t)u8_stage_bytes);
           tma_load_3d(u8 + (size_t)slot * u8_stage_bytes, &tmap, ch0, (int)(t_item + st * kT), 0,
                       &s->u8_full[slot]);
+          if (st % kStep == 0 && it < whole) {
+            // all have come to the step before this one
+            const bool with_all = all_in_step(g.progress, steps++ * gridDim.x, in_step);
+            in_step = in_step && with_all;
+          }
         }
       }
       // drain: every issued copy has landed before the CTA may exit
@@ -884,6 +918,7 @@ cudaError_t launch_gram_tc_pol2(const mraid_plan_s* pl, const uint8_t* d_data, i
   a.R = R;
   a.R2 = R > 16 ? R - 16 : 0;
   a.rb = (R + 1) / 2 * 2;  // B of the first MMAs: R slots, even count
+  a.progress = reinterpret_cast<unsigned*>(pl->d_degenerate + 1);
   a.sums = d_sums;
   a.corr = d_corr;
   a.degenerate = pl->d_degenerate;

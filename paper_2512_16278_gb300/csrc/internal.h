@@ -72,7 +72,7 @@ struct mraid_plan_s {
   int flag_blocks = 0;
   int flag_ctas = 0;                  // widest cluster of the cluster masking kernel (0: none)
   mraid_flag_info* d_info = nullptr;  // device flag info
-  unsigned long long* d_degenerate = nullptr;
+  unsigned long long* d_degenerate = nullptr;  // zero-variance count; [1]: step counter (gram_tc.cu)
   unsigned* d_error = nullptr;        // device error word (bounded waits)
   unsigned long long* d_sweeps = nullptr;  // Jacobi sweeps: [0] per cell, [1] per warp;
                                            // [2] cells whose q1 took the FP64 step

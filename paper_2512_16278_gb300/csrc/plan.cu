@@ -444,7 +444,7 @@ mraid_status mraid_plan(const mraid_params* p, void* stream, mraid_plan_t* out) 
   }
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_partials, sizeof(double) * 6 * (size_t)pl->flag_blocks);
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_info, sizeof(mraid_flag_info));
-  if (e == cudaSuccess) e = cudaMalloc(&pl->d_degenerate, sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc(&pl->d_degenerate, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_error, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_sweeps, 3 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->d_sweeps, 0, 3 * sizeof(unsigned long long), pl->stream);

@@ -135,7 +135,8 @@ mraid_status check_pol2(const mraid_plan_s* pl) {
 // Sums ([cell][P], may be null) and correlation (may be null) of the
 // total power of a two-polarisation block; counts zero-variance beams.
 mraid_status pol2_ccm(mraid_plan_s* pl, const void* d_data, int64_t* d_sums, float* d_corr) {
-  cudaError_t e = cudaMemsetAsync(pl->d_degenerate, 0, sizeof(unsigned long long), pl->stream);
+  // the count, and the step counter of the tensor-core kernel behind it
+  cudaError_t e = cudaMemsetAsync(pl->d_degenerate, 0, 2 * sizeof(unsigned long long), pl->stream);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
   if (pol2_on_tensor_cores(pl, d_data)) {
     e = MRAID_PROF(pl, K_GRAM_TC,

@@ -1,0 +1,53 @@
+"""The two-polarisation Gram takes the same time from call to call (needs a
+GPU). Its CTAs read neighbouring 16-byte pieces of the same lines and are kept
+in step; when they drifted apart, full-size blocks took up to 2.5 times as long
+(6.1 to 15 ms at 13 beams, 8.2 to 17 at 19). The sums of a block with a last
+round of few CTAs equal the CUDA-core Gram's bit for bit."""
+import pytest
+
+from gpu_util import lib
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_beam,n_sub", [(13, 200), (19, 200)])
+def test_steady_time(n_beam, n_sub):
+    import torch
+    m = lib()
+    n_chan, n_s = 4096, 1024
+    part = n_sub * n_s * n_chan
+    d = torch.empty(2 * n_beam * part, dtype=torch.uint8, device="cuda")
+    for b in range(2 * n_beam):
+        d[b * part:(b + 1) * part] = torch.randint(0, 256, (part,), dtype=torch.uint8, device="cuda")
+    with m.Plan(n_beam, n_chan, n_s, n_sub) as plan:
+        corr = torch.empty(plan.n_cells, n_beam * (n_beam + 1) // 2, device="cuda")
+        runs = []
+        for _ in range(41):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            m.mraid_ccm_pol2(plan.handle, d, None, corr)
+            e1.record()
+            torch.cuda.synchronize()
+            runs.append(e0.elapsed_time(e1))
+        plan.sync()
+    runs = sorted(runs[1:])
+    assert runs[35] < 1.15 * runs[0], runs
+    # and near the rate of a block read once (6.1 and 8.2 ms measured)
+    assert runs[20] < 0.55e-3 * n_beam * n_sub / 200 * 1e3, runs
+
+
+@pytest.mark.parametrize("n_chan,n_s,n_sub", [(48, 256, 101), (16, 64, 3), (2432, 128, 2), (2448, 320, 1)])
+def test_rounds_of_few_ctas(n_chan, n_s, n_sub):
+    import torch
+    m = lib()
+    n_beam = 11
+    d = torch.randint(0, 256, (2 * n_beam, n_sub * n_s, n_chan), dtype=torch.uint8, device="cuda")
+    got = {}
+    for variant in (0, -1):
+        with m.Plan(n_beam, n_chan, n_s, n_sub) as plan:
+            m.mraid_set_variant(plan.handle, variant)
+            for _ in range(3):  # the step counter starts anew
+                got[variant] = plan.ccm_pol2(d)
+            plan.sync()
+    assert torch.equal(got[0][0], got[-1][0])
+    assert (got[0][1] - got[-1][1]).abs().max() <= 2e-6
