@@ -235,7 +235,17 @@ mraid_status ccm_range(mraid_plan_s* pl, const void* d_data, int sub0, int n_sub
     }
     return MRAID_OK;
   }
-  const GramRoute route = gram_route(pl, d_data);
+  GramRoute route = gram_route(pl, d_data);
+  if (route != R_MMA && !d_sums && pl->ws.cells < (size_t)cells && !pl->force_dp4a &&
+      gram_mma_supported(pl) && pl->p.n_samp_sub <= kMmPieceMax) {
+    // the faster kernel needs a buffer for its sums that gram_mma does without:
+    // not while the stream is being captured, nor where memory is short
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(pl->stream, &cap);
+    if (e != cudaSuccess) return cuda_fail(e, "capture status");
+    if (cap != cudaStreamCaptureStatusNone || ensure_workspace(pl, (size_t)cells) != MRAID_OK)
+      route = R_MMA;
+  }
   const bool mma = route == R_MMA;
   // profiled by the way the samples come: "gram_tc" for bulk tensor copies
   // ("gram_tcl" above 23 beams), "gram_u8" for plain ones; mraid_gram_kernel
