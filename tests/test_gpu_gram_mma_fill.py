@@ -46,6 +46,7 @@ def test_no_sample_is_copied_twice():
             runs = []
             for _ in range(8):
                 e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                torch.cuda._sleep(100000)
                 e0.record()
                 m.mraid_ccm(plan.handle, d, None, corr)
                 e1.record()

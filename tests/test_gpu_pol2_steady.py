@@ -24,6 +24,7 @@ def test_steady_time(n_beam, n_sub):
         runs = []
         for _ in range(41):
             e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda._sleep(1_000_000)  # the launch is queued before the clock starts
             e0.record()
             m.mraid_ccm_pol2(plan.handle, d, None, corr)
             e1.record()

@@ -28,7 +28,7 @@ def test_a_short_block_times_out_once(n_beam, stage):
             plan.sync()
         took = time.monotonic() - t0
         assert e.value.status == 5
-        assert limit * 0.9 < took < 2.5 * limit, took
+        assert limit * 0.9 < took < 4 * limit, took
         corr = plan.ccm(d, sums=False)[1]
         plan.sync()
         assert torch.equal(corr.cpu(), ref)
